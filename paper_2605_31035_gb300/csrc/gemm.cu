@@ -264,7 +264,7 @@ mixfp4_gemm_kernel(const __grid_constant__ CUtensorMap tm_ac, const __grid_const
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       tma_prefetch(&tm_ac);
       tma_prefetch(&tm_bc);
       tma_prefetch(&tm_as);
@@ -310,7 +310,7 @@ mixfp4_gemm_kernel(const __grid_constant__ CUtensorMap tm_ac, const __grid_const
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (leader CTA) ----------------
-    if (leader && lane == 0) {
+    if (leader && elect_one()) {
       int d = 0;
       uint32_t dph = 0;
       bool ok = true;
@@ -460,6 +460,7 @@ mixfp4_gemm_kernel(const __grid_constant__ CUtensorMap tm_ac, const __grid_const
     // 16-byte aligned) each lane stores its row's 16 values one by one.
     const int q = warp & 3;                  // TMEM lane quarter of this warp
     const int chalf = (warp - kFirstEpi) >> 2;  // column half
+    const bool elected = elect_one();
     griddep_wait();
     const float sa = 0.25f * __ldg(a_ts), sb = __ldg(b_ts);
     const u64 sa2 = pack2(sa, sa), sb2 = pack2(sb, sb);
@@ -484,7 +485,7 @@ mixfp4_gemm_kernel(const __grid_constant__ CUtensorMap tm_ac, const __grid_const
       // An add into C must follow the earlier segments' stores into the same
       // tile: bulk operations of different groups are not ordered, so wait
       // for their completion (issued a main loop ago, they are done).
-      if (!whole && c_tma && lane == 0) bulk_wait_all();
+      if (!whole && c_tma && elected) bulk_wait_all();
       const bool acc_ok = mbar_wait_cluster(smem_u32(&bars->acc_full), i & 1, abort_flag, wait_ns);
       tc_fence_after();
       // tcgen05.ld is warp-collective: decide for the whole warp.
@@ -518,7 +519,7 @@ mixfp4_gemm_kernel(const __grid_constant__ CUtensorMap tm_ac, const __grid_const
         if (c_tma) {
           const uint32_t stage = (kTwoStages && (cc & 1)) ? stage1 : stage0;
           // The store that last used this staging tile must have read it.
-          if (lane == 0) {
+          if (elected) {
             if (kTwoStages) bulk_wait_read_one();
             else bulk_wait_read_all();
           }
@@ -529,7 +530,7 @@ mixfp4_gemm_kernel(const __grid_constant__ CUtensorMap tm_ac, const __grid_const
                    o[4 * j + 3]);
           fence_proxy_async_smem();
           __syncwarp();
-          if (lane == 0) {
+          if (elected) {
             if (row0 < M && col < N) {  // boxes wholly outside C are skipped
               if (whole) tma_store_2d(&tm_c, stage, col, row0);
               else tma_reduce_add_2d(&tm_c, stage, col, row0);
@@ -547,7 +548,7 @@ mixfp4_gemm_kernel(const __grid_constant__ CUtensorMap tm_ac, const __grid_const
       }
     }
     // The CTA's stores into C complete before it exits.
-    if (c_tma && lane == 0) bulk_wait_all();
+    if (c_tma && elected) bulk_wait_all();
   }
 
   tc_fence_before();
@@ -676,7 +677,7 @@ mixfp4_gemm_skinny_kernel(const __grid_constant__ CUtensorMap tm_wc, const __gri
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       tma_prefetch(&tm_wc);
       tma_prefetch(&tm_xc);
       tma_prefetch(&tm_ws);
@@ -709,7 +710,7 @@ mixfp4_gemm_skinny_kernel(const __grid_constant__ CUtensorMap tm_wc, const __gri
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       int d = 0, ntile = 0;
       uint32_t dph = 0;
       bool ok = true;

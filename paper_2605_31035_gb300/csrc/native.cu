@@ -225,7 +225,7 @@ nvf4_gemm_kernel(const __grid_constant__ CUtensorMap tm_am, const __grid_constan
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       tma_prefetch(&tm_am);
       tma_prefetch(&tm_bm);
       if (kARes) tma_prefetch(&tm_ar);
@@ -271,7 +271,7 @@ nvf4_gemm_kernel(const __grid_constant__ CUtensorMap tm_am, const __grid_constan
       }
     }
   } else if (warp == 1) {
-    if (leader && lane == 0) {
+    if (leader && elect_one()) {
       // ---------------- MMA issuer ----------------
       constexpr uint32_t kIdesc = idesc_nvf4_f32(TILE_M, TILE_N);
       int it = 0;
@@ -640,7 +640,7 @@ nvf4_fewrows_kernel(const __grid_constant__ CUtensorMap tm_wc, const __grid_cons
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       tma_prefetch(&tm_wc);
       tma_prefetch(&tm_ws);
       tma_prefetch(&tm_xc);
@@ -671,7 +671,7 @@ nvf4_fewrows_kernel(const __grid_constant__ CUtensorMap tm_wc, const __grid_cons
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t kIdesc = idesc_nvf4_f32(128, 2 * WR);
       int it = 0, run = 0;
       bool ok = true;
@@ -717,7 +717,7 @@ nvf4_fewrows_kernel(const __grid_constant__ CUtensorMap tm_wc, const __grid_cons
     // stage's columns are rewritten only after its next TMA landing, which
     // follows the MMAs that read them.
     const int j0 = 2 * (warp - kCopyWarp);
-    if (lane == 0) {
+    if (elect_one()) {
       int it = 0;
       for (long long u = u_begin; u < u_end; ++u, ++it) {
         const int s = it % NST;
