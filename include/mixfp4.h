@@ -291,6 +291,24 @@ int mixfp4_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_
                 uint32_t* status_word, void* stream);
 
 /*
+ * mixfp4_linear -- the W4A4 linear layer in one call: Algorithm 1 on the
+ * activations (mixfp4_quantize with MIXFP4_SCALE_COMPUTE) into scratch memory,
+ * then C = X_deq . W_deq^T (mixfp4_gemm).
+ *
+ * x, dtype, M, K, ldx, mode  as mixfp4_quantize's x, dtype, rows, K, ldx, mode, with
+ *              K % 256 == 0 as mixfp4_gemm's.
+ * w_codes/w_scales/w_ts      W, N x K, as mixfp4_gemm's B.
+ * C, ldc, status_word        as mixfp4_gemm's.
+ * workspace    device, 256-byte aligned, at least 2 M K + 512 bytes; written by the
+ *              call and free for reuse once the call's work on `stream` is done.
+ * workspace_bytes  its size.
+ */
+int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, int mode,
+                  const uint8_t* w_codes, const uint8_t* w_scales, const float* w_ts, int64_t N,
+                  float* C, int64_t ldc, void* workspace, int64_t workspace_bytes,
+                  uint32_t* status_word, void* stream);
+
+/*
  * mixfp4_split_native -- the operands of the native FP4 GEMM variant.  A
  * MixFP4 tensor is rewritten as the sum of two E2M1 tensors that share its
  * block scales (no counterpart in the paper; every value is exact):

@@ -319,6 +319,28 @@ int mixfp4_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_
   return launch_status();
 }
 
+int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, int mode, const uint8_t* w_codes,
+                  const uint8_t* w_scales, const float* w_ts, int64_t N, float* C, int64_t ldc, void* workspace,
+                  int64_t workspace_bytes, uint32_t* status_word, void* stream) {
+  if (M < 0 || N < 0 || K < 0 || K % 256 != 0 || ldx < K || ldc < N) return MIXFP4_ERR_SHAPE;
+  if (M == 0 || N == 0 || K == 0) {  // no activations to quantize, or nothing to reduce
+    if (dtype != MIXFP4_DTYPE_BF16) return MIXFP4_ERR_DTYPE;
+    if (mode < MIXFP4_MODE_MIX || mode > MIXFP4_MODE_FOUR_SIX) return MIXFP4_ERR_ARG;
+    return mixfp4_gemm(nullptr, nullptr, nullptr, w_codes, w_scales, w_ts, M, N, K, C, ldc, status_word, stream);
+  }
+  if (!workspace) return MIXFP4_ERR_NULL;
+  if (!aligned(workspace, 256)) return MIXFP4_ERR_ALIGN;
+  if (M > (1 << 30) || N > (1 << 30) || K > (1 << 30) || workspace_bytes < 2 * M * K + 512) return MIXFP4_ERR_SHAPE;
+  // Scratch: the amax word and s32, then the codes, then the block scales.
+  uint32_t* amax_word = static_cast<uint32_t*>(workspace);
+  float* x_ts = static_cast<float*>(workspace) + 4;
+  uint8_t* codes = static_cast<uint8_t*>(workspace) + 256;
+  uint8_t* scales = codes + M * (K / 2);  // K / 2 is a multiple of 128
+  if (int st = mixfp4_quantize(x, dtype, M, K, ldx, codes, scales, x_ts, amax_word, mode, MIXFP4_SCALE_COMPUTE, stream))
+    return st;
+  return mixfp4_gemm(codes, scales, x_ts, w_codes, w_scales, w_ts, M, N, K, C, ldc, status_word, stream);
+}
+
 int mixfp4_gemm_native_fewrows(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts,
                                const uint8_t* b_codes, const uint8_t* b_scales, const float* b_ts, int64_t M,
                                int64_t N, int64_t K, float* C, int64_t ldc, uint32_t* status_word, void* stream) {

@@ -21,6 +21,8 @@ CAND_E2M1_6, CAND_E1M2, CAND_E2M1_4, CAND_E3M0 = 1, 2, 4, 8
 STATUS = {0: "ok", -1: "null pointer", -2: "invalid shape", -3: "misaligned", -4: "unsupported dtype",
           -5: "CUDA error", -6: "device-side wait timed out", -7: "argument out of range"}
 
+_ERR_CUDA = -5
+
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libmixfp4.so")
 _lib = None
 
@@ -61,6 +63,8 @@ def lib() -> ctypes.CDLL:
         L.mixfp4_dequantize.argtypes = [P, P, P, I64, I64, P, P]
         L.mixfp4_gemm.restype = I
         L.mixfp4_gemm.argtypes = [P, P, P, P, P, P, I64, I64, I64, P, I64, P, P]
+        L.mixfp4_linear.restype = I
+        L.mixfp4_linear.argtypes = [P, I, I64, I64, I64, I, P, P, P, I64, P, I64, P, I64, P, P]
         L.mixfp4_split_native.restype = I
         L.mixfp4_split_native.argtypes = [P, P, I64, I64, P, P, P, P]
         L.mixfp4_gemm_native.restype = I
@@ -88,9 +92,14 @@ def _require(cond: bool, msg: str):
         raise ValueError(msg)
 
 
+# The checks below build their messages only when they fail: a call on a few
+# rows takes less time on the GPU than formatting them takes on the host.
+
+
 def _check_x(x: torch.Tensor):
-    _require(isinstance(x, torch.Tensor) and x.is_cuda and x.dtype == torch.bfloat16 and x.dim() == 2
-             and x.stride(1) == 1, "x must be a 2-D bf16 CUDA tensor with unit column stride")
+    if not (isinstance(x, torch.Tensor) and x.is_cuda and x.dtype is torch.bfloat16 and x.dim() == 2
+            and x.stride(1) == 1):
+        raise ValueError("x must be a 2-D bf16 CUDA tensor with unit column stride")
 
 
 def _check_signs(signs):
@@ -100,42 +109,45 @@ def _check_signs(signs):
 
 def _check_dev(t, device, what: str):
     """t must be a CUDA tensor on `device` (the device of the call's main input)."""
-    _require(isinstance(t, torch.Tensor) and t.is_cuda and t.device == device,
-             f"{what} must be a CUDA tensor on {device}")
+    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.device == device):
+        raise ValueError(f"{what} must be a CUDA tensor on {device}")
 
 
 def _check_u8(t, shape, device, what: str):
     _check_dev(t, device, what)
-    _require(t.dtype == torch.uint8 and tuple(t.shape) == tuple(shape) and t.is_contiguous(),
-             f"{what} must be a dense uint8 tensor of shape {tuple(shape)}")
+    if not (t.dtype is torch.uint8 and t.shape == shape and t.is_contiguous()):
+        raise ValueError(f"{what} must be a dense uint8 tensor of shape {tuple(shape)}")
 
 
 def _check_scalar_f32(t, device, what: str):
     _check_dev(t, device, what)
-    _require(t.dtype == torch.float32 and t.numel() >= 1, f"{what} must hold at least one float32")
+    if not (t.dtype is torch.float32 and t.numel() >= 1):
+        raise ValueError(f"{what} must hold at least one float32")
 
 
 def _check_qtensor(q, rows: int, K: int, device, what: str):
     """A MixFP4 operand: codes uint8 [rows, K/2], scales uint8 [rows, K/16], s32 float32, all on `device`."""
-    _require(isinstance(q, QTensor), f"{what} must be a QTensor")
-    _check_u8(q.codes, (rows, K // 2), device, f"{what}.codes")
-    _check_u8(q.scales, (rows, K // 16), device, f"{what}.scales")
-    _check_scalar_f32(q.tensor_scale, device, f"{what}.tensor_scale")
+    if not isinstance(q, QTensor):
+        raise ValueError(f"{what} must be a QTensor")
+    _check_u8(q.codes, (rows, K // 2), device, what + ".codes")
+    _check_u8(q.scales, (rows, K // 16), device, what + ".scales")
+    _check_scalar_f32(q.tensor_scale, device, what + ".tensor_scale")
 
 
 def _check_operand(q, what: str):
     """A GEMM operand: a QTensor on a CUDA device, consistent with its own codes shape."""
-    _require(isinstance(q, QTensor) and isinstance(q.codes, torch.Tensor) and q.codes.dim() == 2,
-             f"{what} must be a QTensor with 2-D codes")
-    _check_qtensor(q, q.rows, q.K, q.codes.device, what)
+    if not (isinstance(q, QTensor) and isinstance(q.codes, torch.Tensor) and q.codes.dim() == 2):
+        raise ValueError(f"{what} must be a QTensor with 2-D codes")
+    rows, half = q.codes.shape
+    _check_qtensor(q, rows, half * 2, q.codes.device, what)
 
 
 def _check_c(C, M: int, N: int, device):
     """GEMM output: float32 [M, N] on `device`, unit column stride (row stride >= N)."""
     _check_dev(C, device, "out")
-    _require(C.dtype == torch.float32 and C.dim() == 2 and tuple(C.shape) == (M, N)
-             and (C.stride(1) == 1 or N <= 1) and C.stride(0) >= max(N, 1),
-             f"out must be a float32 [{M}, {N}] tensor with unit column stride")
+    if not (C.dtype is torch.float32 and C.dim() == 2 and C.shape == (M, N)
+            and (C.stride(1) == 1 or N <= 1) and C.stride(0) >= max(N, 1)):
+        raise ValueError(f"out must be a float32 [{M}, {N}] tensor with unit column stride")
 
 
 def _check_workspace(ws, device):
@@ -158,12 +170,13 @@ def _check_given_scale(ts):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _check(fn: str, status: int):
@@ -187,10 +200,37 @@ class QTensor:
         return self.codes.shape[1] * 2
 
 
+def _scratch(nbytes: int, device):
+    """Scratch memory that a call takes and returns, or None where the device
+    has no room for it (the caller then goes without)."""
+    try:
+        return torch.empty(nbytes, dtype=torch.uint8, device=device)
+    except torch.OutOfMemoryError:
+        return None
+
+
 def empty_qtensor(rows: int, K: int, device) -> QTensor:
     return QTensor(torch.empty(rows, K // 2, dtype=torch.uint8, device=device),
                    torch.empty(rows, K // 16, dtype=torch.uint8, device=device),
                    torch.empty(1, dtype=torch.float32, device=device))
+
+
+def _quantizer_args(x, rows: int, K: int, tensor_scale, out, workspace):
+    """Outputs and scratch of a quantizer call whose result is [rows, K]:
+    (QTensor, workspace or None, scale flag)."""
+    if out is None:
+        q = empty_qtensor(rows, K, x.device)
+    else:
+        q = out
+        _check_qtensor(q, rows, K, x.device, "out")
+    if tensor_scale is not None:
+        _check_given_scale(tensor_scale)
+        q.tensor_scale.copy_(tensor_scale.reshape(1))
+        return q, None, SCALE_GIVEN
+    if workspace is None:
+        return q, torch.empty(1, dtype=torch.int32, device=x.device), SCALE_COMPUTE
+    _check_workspace(workspace, x.device)
+    return q, workspace, SCALE_COMPUTE
 
 
 def mixfp4_quantize(x: torch.Tensor, mode: int = MODE_MIX, tensor_scale: torch.Tensor | None = None,
@@ -203,19 +243,9 @@ def mixfp4_quantize(x: torch.Tensor, mode: int = MODE_MIX, tensor_scale: torch.T
     """
     _check_x(x)
     rows, K = x.shape
-    q = out if out is not None else empty_qtensor(rows, K, x.device)
-    _check_qtensor(q, rows, K, x.device, "out")
-    _check_given_scale(tensor_scale)
-    given = tensor_scale is not None
-    if given:
-        q.tensor_scale.copy_(tensor_scale.reshape(1))
-    ws = None
-    if not given:
-        ws = workspace if workspace is not None else torch.empty(1, dtype=torch.int32, device=x.device)
-        _check_workspace(ws, x.device)
+    q, ws, flag = _quantizer_args(x, rows, K, tensor_scale, out, workspace)
     st = lib().mixfp4_quantize(_ptr(x), DTYPE_BF16, rows, K, x.stride(0), _ptr(q.codes), _ptr(q.scales),
-                               _ptr(q.tensor_scale), _ptr(ws), int(mode),
-                               SCALE_GIVEN if given else SCALE_COMPUTE, _stream(stream))
+                               _ptr(q.tensor_scale), _ptr(ws), int(mode), flag, _stream(stream))
     _check("mixfp4_quantize", st)
     return q
 
@@ -229,19 +259,10 @@ def mixfp4_quantize_rht(x: torch.Tensor, signs: torch.Tensor | None = None, mode
     _check_x(x)
     _check_signs(signs)
     rows, K = x.shape
-    q = out if out is not None else empty_qtensor(rows, K, x.device)
-    _check_qtensor(q, rows, K, x.device, "out")
-    _check_given_scale(tensor_scale)
-    given = tensor_scale is not None
-    if given:
-        q.tensor_scale.copy_(tensor_scale.reshape(1))
-    ws = None
-    if not given:
-        ws = workspace if workspace is not None else torch.empty(1, dtype=torch.int32, device=x.device)
-        _check_workspace(ws, x.device)
+    q, ws, flag = _quantizer_args(x, rows, K, tensor_scale, out, workspace)
     st = lib().mixfp4_quantize_rht(_ptr(x), DTYPE_BF16, rows, K, x.stride(0), _ptr(signs), _ptr(q.codes),
-                                   _ptr(q.scales), _ptr(q.tensor_scale), _ptr(ws), int(mode),
-                                   SCALE_GIVEN if given else SCALE_COMPUTE, _stream(stream))
+                                   _ptr(q.scales), _ptr(q.tensor_scale), _ptr(ws), int(mode), flag,
+                                   _stream(stream))
     _check("mixfp4_quantize_rht", st)
     return q
 
@@ -254,19 +275,9 @@ def mixfp4_quantize_colwise(x: torch.Tensor, mode: int = MODE_MIX, tensor_scale:
     X^T, codes [C, R/2], scales [C, R/16]."""
     _check_x(x)
     R, C = x.shape
-    q = out if out is not None else empty_qtensor(C, R, x.device)
-    _check_qtensor(q, C, R, x.device, "out")
-    _check_given_scale(tensor_scale)
-    given = tensor_scale is not None
-    if given:
-        q.tensor_scale.copy_(tensor_scale.reshape(1))
-    ws = None
-    if not given:
-        ws = workspace if workspace is not None else torch.empty(1, dtype=torch.int32, device=x.device)
-        _check_workspace(ws, x.device)
+    q, ws, flag = _quantizer_args(x, C, R, tensor_scale, out, workspace)
     st = lib().mixfp4_quantize_colwise(_ptr(x), DTYPE_BF16, R, C, x.stride(0), _ptr(q.codes), _ptr(q.scales),
-                                       _ptr(q.tensor_scale), _ptr(ws), int(mode),
-                                       SCALE_GIVEN if given else SCALE_COMPUTE, _stream(stream))
+                                       _ptr(q.tensor_scale), _ptr(ws), int(mode), flag, _stream(stream))
     _check("mixfp4_quantize_colwise", st)
     return q
 
@@ -279,19 +290,10 @@ def mixfp4_quantize_colwise_rht(x: torch.Tensor, signs: torch.Tensor | None = No
     _check_x(x)
     _check_signs(signs)
     R, C = x.shape
-    q = out if out is not None else empty_qtensor(C, R, x.device)
-    _check_qtensor(q, C, R, x.device, "out")
-    _check_given_scale(tensor_scale)
-    given = tensor_scale is not None
-    if given:
-        q.tensor_scale.copy_(tensor_scale.reshape(1))
-    ws = None
-    if not given:
-        ws = workspace if workspace is not None else torch.empty(1, dtype=torch.int32, device=x.device)
-        _check_workspace(ws, x.device)
+    q, ws, flag = _quantizer_args(x, C, R, tensor_scale, out, workspace)
     st = lib().mixfp4_quantize_colwise_rht(_ptr(x), DTYPE_BF16, R, C, x.stride(0), _ptr(signs), _ptr(q.codes),
-                                           _ptr(q.scales), _ptr(q.tensor_scale), _ptr(ws), int(mode),
-                                           SCALE_GIVEN if given else SCALE_COMPUTE, _stream(stream))
+                                           _ptr(q.scales), _ptr(q.tensor_scale), _ptr(ws), int(mode), flag,
+                                           _stream(stream))
     _check("mixfp4_quantize_colwise_rht", st)
     return q
 
@@ -303,20 +305,10 @@ def mixfp4_quantize_sr(x: torch.Tensor, seed: int, offset: int = 0, mode: int = 
     stochastic rounding of the codes drawn from (seed, offset)."""
     _check_x(x)
     rows, K = x.shape
-    q = out if out is not None else (empty_qtensor(K, rows, x.device) if colwise else empty_qtensor(rows, K, x.device))
-    _check_qtensor(q, K if colwise else rows, rows if colwise else K, x.device, "out")
-    _check_given_scale(tensor_scale)
-    given = tensor_scale is not None
-    if given:
-        q.tensor_scale.copy_(tensor_scale.reshape(1))
-    ws = None
-    if not given:
-        ws = workspace if workspace is not None else torch.empty(1, dtype=torch.int32, device=x.device)
-        _check_workspace(ws, x.device)
+    q, ws, flag = _quantizer_args(x, K if colwise else rows, rows if colwise else K, tensor_scale, out, workspace)
     fn = lib().mixfp4_quantize_colwise_sr if colwise else lib().mixfp4_quantize_sr
     st = fn(_ptr(x), DTYPE_BF16, rows, K, x.stride(0), _ptr(q.codes), _ptr(q.scales), _ptr(q.tensor_scale),
-            _ptr(ws), int(mode), SCALE_GIVEN if given else SCALE_COMPUTE, int(seed) & (2 ** 64 - 1),
-            int(offset) & (2 ** 64 - 1), _stream(stream))
+            _ptr(ws), int(mode), flag, int(seed) & (2 ** 64 - 1), int(offset) & (2 ** 64 - 1), _stream(stream))
     _check("mixfp4_quantize_colwise_sr" if colwise else "mixfp4_quantize_sr", st)
     return q
 
@@ -328,19 +320,9 @@ def mixfp4_quantize_2d(x: torch.Tensor, mode: int = MODE_MIX, tensor_scale: torc
     and format per tile, repeated on the tile's rows)."""
     _check_x(x)
     rows, K = x.shape
-    q = out if out is not None else empty_qtensor(rows, K, x.device)
-    _check_qtensor(q, rows, K, x.device, "out")
-    _check_given_scale(tensor_scale)
-    given = tensor_scale is not None
-    if given:
-        q.tensor_scale.copy_(tensor_scale.reshape(1))
-    ws = None
-    if not given:
-        ws = workspace if workspace is not None else torch.empty(1, dtype=torch.int32, device=x.device)
-        _check_workspace(ws, x.device)
+    q, ws, flag = _quantizer_args(x, rows, K, tensor_scale, out, workspace)
     st = lib().mixfp4_quantize_2d(_ptr(x), DTYPE_BF16, rows, K, x.stride(0), _ptr(q.codes), _ptr(q.scales),
-                                  _ptr(q.tensor_scale), _ptr(ws), int(mode),
-                                  SCALE_GIVEN if given else SCALE_COMPUTE, _stream(stream))
+                                  _ptr(q.tensor_scale), _ptr(ws), int(mode), flag, _stream(stream))
     _check("mixfp4_quantize_2d", st)
     return q
 
@@ -349,11 +331,13 @@ def mixfp4_transpose_2d(q: QTensor, out: QTensor | None = None, stream=None) -> 
     """The transpose of a 2D-quantized tensor (rows and K multiples of 16);
     the tensor scale is shared with the input."""
     _check_operand(q, "q")
-    t = out if out is not None else QTensor(
-        torch.empty(q.K, q.rows // 2, dtype=torch.uint8, device=q.codes.device),
-        torch.empty(q.K, q.rows // 16, dtype=torch.uint8, device=q.codes.device), q.tensor_scale)
-    _check_u8(t.codes, (q.K, q.rows // 2), q.codes.device, "out.codes")
-    _check_u8(t.scales, (q.K, q.rows // 16), q.codes.device, "out.scales")
+    if out is None:
+        t = QTensor(torch.empty(q.K, q.rows // 2, dtype=torch.uint8, device=q.codes.device),
+                    torch.empty(q.K, q.rows // 16, dtype=torch.uint8, device=q.codes.device), q.tensor_scale)
+    else:
+        t = out
+        _check_u8(t.codes, (q.K, q.rows // 2), q.codes.device, "out.codes")
+        _check_u8(t.scales, (q.K, q.rows // 16), q.codes.device, "out.scales")
     st = lib().mixfp4_transpose_2d(_ptr(q.codes), _ptr(q.scales), q.rows, q.K, _ptr(t.codes), _ptr(t.scales),
                                    _stream(stream))
     _check("mixfp4_transpose_2d", st)
@@ -412,6 +396,13 @@ def mixfp4_dequantize(q: QTensor, out: torch.Tensor | None = None, stream=None) 
     return o
 
 
+def _gemm_out(out, M: int, N: int, device):
+    if out is None:
+        return torch.empty(M, N, dtype=torch.float32, device=device)
+    _check_c(out, M, N, device)
+    return out
+
+
 def mixfp4_gemm(a: QTensor, b: QTensor, out: torch.Tensor | None = None,
                 status_word: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """C = A_deq . B_deq^T in fp32; a is M x K, b is N x K."""
@@ -419,8 +410,7 @@ def mixfp4_gemm(a: QTensor, b: QTensor, out: torch.Tensor | None = None,
     _check_operand(b, "b")
     _require(a.K == b.K and a.codes.device == b.codes.device, "operands must share K and device")
     M, N, K = a.rows, b.rows, a.K
-    C = out if out is not None else torch.empty(M, N, dtype=torch.float32, device=a.codes.device)
-    _check_c(C, M, N, a.codes.device)
+    C = _gemm_out(out, M, N, a.codes.device)
     _check_status(status_word, a.codes.device)
     st = lib().mixfp4_gemm(_ptr(a.codes), _ptr(a.scales), _ptr(a.tensor_scale),
                            _ptr(b.codes), _ptr(b.scales), _ptr(b.tensor_scale),
@@ -454,13 +444,13 @@ def sf_tiled_bytes(rows: int, K: int) -> int:
 
 def _check_native(t, rows: int, K: int, device, what: str):
     """Native operand: main (and residual, if any) uint8 [rows, K/2], tiled scales, s32, all on `device`."""
-    _check_u8(t.main, (rows, K // 2), device, f"{what}.main")
+    _check_u8(t.main, (rows, K // 2), device, what + ".main")
     if t.res is not None:
-        _check_u8(t.res, (rows, K // 2), device, f"{what}.res")
-    _check_dev(t.sf, device, f"{what}.sf")
-    _require(t.sf.dtype == torch.uint8 and t.sf.is_contiguous() and t.sf.numel() >= sf_tiled_bytes(rows, K),
-             f"{what}.sf must be a dense uint8 buffer of at least {sf_tiled_bytes(rows, K)} bytes")
-    _check_scalar_f32(t.tensor_scale, device, f"{what}.tensor_scale")
+        _check_u8(t.res, (rows, K // 2), device, what + ".res")
+    _check_dev(t.sf, device, what + ".sf")
+    if not (t.sf.dtype is torch.uint8 and t.sf.is_contiguous() and t.sf.numel() >= sf_tiled_bytes(rows, K)):
+        raise ValueError(f"{what}.sf must be a dense uint8 buffer of at least {sf_tiled_bytes(rows, K)} bytes")
+    _check_scalar_f32(t.tensor_scale, device, what + ".tensor_scale")
 
 
 def mixfp4_split_native(q: QTensor, keep_residual: bool = True, out: NativeTensor | None = None,
@@ -494,8 +484,7 @@ def mixfp4_gemm_native(a: NativeTensor, b: NativeTensor, out: torch.Tensor | Non
     _check_native(b, b.rows, b.K, dev, "b")
     _require(a.K == b.K, "operands must share K")
     M, N, K = a.rows, b.rows, a.K
-    C = out if out is not None else torch.empty(M, N, dtype=torch.float32, device=a.main.device)
-    _check_c(C, M, N, dev)
+    C = _gemm_out(out, M, N, dev)
     _check_status(status_word, dev)
     st = lib().mixfp4_gemm_native(_ptr(a.main), _ptr(a.res), _ptr(a.sf), _ptr(a.tensor_scale),
                                   _ptr(b.main), _ptr(b.res), _ptr(b.sf), _ptr(b.tensor_scale),
@@ -514,8 +503,7 @@ def mixfp4_gemm_native_fewrows(a: QTensor, b: QTensor, out: torch.Tensor | None 
     _require(a.K == b.K and a.rows <= 64 and a.codes.device == b.codes.device,
              "operands must share K and device, and A have at most 64 rows")
     M, N, K = a.rows, b.rows, a.K
-    C = out if out is not None else torch.empty(M, N, dtype=torch.float32, device=a.codes.device)
-    _check_c(C, M, N, a.codes.device)
+    C = _gemm_out(out, M, N, a.codes.device)
     _check_status(status_word, a.codes.device)
     st = lib().mixfp4_gemm_native_fewrows(_ptr(a.codes), _ptr(a.scales), _ptr(a.tensor_scale),
                                           _ptr(b.codes), _ptr(b.scales), _ptr(b.tensor_scale),
@@ -555,4 +543,22 @@ def selftest_gemm_missed_stage(a: QTensor, b: QTensor, out: torch.Tensor, limit_
 def linear(x: torch.Tensor, w_q: QTensor, mode: int = MODE_MIX, stream=None) -> torch.Tensor:
     """W4A4 linear: quantize the activations online, then the MixFP4 GEMM with
     pre-quantized weights.  Returns x_deq . w_deq^T in fp32."""
+    _check_x(x)
+    M, K = x.shape
+    if M > 0 and K > 0 and isinstance(w_q, QTensor) and isinstance(w_q.codes, torch.Tensor) \
+            and w_q.codes.dim() == 2 and w_q.codes.shape[1] * 2 == K and w_q.codes.device == x.device:
+        _check_operand(w_q, "b")
+        N = w_q.codes.shape[0]
+        C = torch.empty(M, N, dtype=torch.float32, device=x.device)
+        ws = _scratch(2 * M * K + 512, x.device)
+        if ws is not None:
+            st = lib().mixfp4_linear(_ptr(x), DTYPE_BF16, M, K, x.stride(0), int(mode), _ptr(w_q.codes),
+                                     _ptr(w_q.scales), _ptr(w_q.tensor_scale), N, _ptr(C), N, _ptr(ws), ws.numel(),
+                                     None, _stream(stream))
+            if stream is not None:
+                ws.record_stream(stream)  # allocated on the current stream, used on the caller's
+            if st in (0, _ERR_CUDA):
+                _check("mixfp4_linear", st)
+                return C
+            # Refused, with nothing enqueued: the two calls below say which one refuses it, and why.
     return mixfp4_gemm(mixfp4_quantize(x, mode, stream=stream), w_q, stream=stream)
