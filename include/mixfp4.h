@@ -301,12 +301,50 @@ int mixfp4_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_
  * C, ldc, status_word        as mixfp4_gemm's.
  * workspace    device, 256-byte aligned, at least 2 M K + 512 bytes; written by the
  *              call and free for reuse once the call's work on `stream` is done.
+ *              With the bytes mixfp4_linear_workspace reports, a long K may be cut
+ *              into parts that run side by side (their sum is compensated).
  * workspace_bytes  its size.
  */
 int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, int mode,
                   const uint8_t* w_codes, const uint8_t* w_scales, const float* w_ts, int64_t N,
                   float* C, int64_t ldc, void* workspace, int64_t workspace_bytes,
                   uint32_t* status_word, void* stream);
+
+/*
+ * mixfp4_linear_workspace -- bytes of workspace mixfp4_linear makes use of, at
+ * least the 2 M K + 512 it needs, on the current device.
+ *
+ * bytes        host, one int64.                                          (output)
+ */
+int mixfp4_linear_workspace(int64_t M, int64_t N, int64_t K, int64_t* bytes);
+
+/*
+ * mixfp4_gemm_ws -- mixfp4_gemm with scratch memory.  With `workspace_bytes`
+ * >= the bytes mixfp4_gemm_workspace reports (and those positive) A is first decoded
+ * to f16 in the workspace (App. B.5 values times the block scales, exact), so
+ * the main loop decodes only B, and a long K may be cut into parts that run
+ * side by side (their sum is compensated); otherwise, and with workspace = NULL, the call
+ * is mixfp4_gemm.
+ *
+ * workspace       device, 256-byte aligned, or NULL; written by the call and free
+ *                 for reuse once the call's work on `stream` is done.
+ * workspace_bytes its size.
+ * The other arguments are mixfp4_gemm's.
+ */
+int mixfp4_gemm_ws(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts,
+                   const uint8_t* b_codes, const uint8_t* b_scales, const float* b_ts,
+                   int64_t M, int64_t N, int64_t K, float* C, int64_t ldc,
+                   void* workspace, int64_t workspace_bytes,
+                   uint32_t* status_word, void* stream);
+
+/*
+ * mixfp4_gemm_workspace -- bytes of device workspace mixfp4_gemm_ws wants for
+ * an M x N x K product of MixFP4 operands (App. B.1) on the current device;
+ * 0 when it takes none.  Sizes are checked as mixfp4_gemm's.
+ *
+ * bytes        host, one int64.                                          (output)
+ */
+int mixfp4_gemm_workspace(int64_t M, int64_t N, int64_t K, int64_t* bytes);
 
 /*
  * mixfp4_split_native -- the operands of the native FP4 GEMM variant.  A

@@ -291,10 +291,20 @@ int mixfp4_dequantize(const uint8_t* codes, const uint8_t* scales, const float* 
   return launch_status();
 }
 
-int mixfp4_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts,
-                const uint8_t* b_codes, const uint8_t* b_scales, const float* b_ts,
-                int64_t M, int64_t N, int64_t K, float* C, int64_t ldc,
-                uint32_t* status_word, void* stream) {
+namespace {
+
+// Workspace of mixfp4_gemm_ws: A decoded to f16 where that pays (2 M K bytes, a
+// multiple of 512), then the parts of a split K.
+int64_t gemm_scratch(int64_t M, int64_t N, int64_t K) {
+  if (M <= 64 || N <= 0 || K <= 0 || M > (1 << 30) || N > (1 << 30) || K > (1 << 30)) return 0;
+  if (!mixfp4::gemm_predecode_pays(M, N, K)) return 0;
+  return M * K * 2 + mixfp4::gemm_f16a_parts_bytes(M, N, K);
+}
+
+// Shared body of the decode-path GEMM entry points.
+int gemm_impl(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts, const uint8_t* b_codes,
+              const uint8_t* b_scales, const float* b_ts, int64_t M, int64_t N, int64_t K, float* C, int64_t ldc,
+              void* workspace, int64_t workspace_bytes, uint32_t* status_word, void* stream) {
   if (M < 0 || N < 0 || K < 0 || K % 256 != 0 || ldc < N) return MIXFP4_ERR_SHAPE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (status_word) {
@@ -313,10 +323,52 @@ int mixfp4_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_
   if (!aligned(a_codes, 16) || !aligned(a_scales, 16) || !aligned(b_codes, 16) ||
       !aligned(b_scales, 16) || !aligned(a_ts, 4) || !aligned(b_ts, 4))
     return MIXFP4_ERR_ALIGN;
-  int st = mixfp4::launch_gemm(a_codes, a_scales, a_ts, b_codes, b_scales, b_ts, M, N, K, C, ldc,
-                               status_word, s);
+  const int64_t need = gemm_scratch(M, N, K);
+  int st;
+  if (need > 0 && workspace && workspace_bytes >= need) {
+    if (!aligned(workspace, 256)) return MIXFP4_ERR_ALIGN;
+    if (mixfp4::launch_decode_f16(a_codes, a_scales, M, K, workspace, s) != 0) return MIXFP4_ERR_CUDA;
+    st = mixfp4::launch_gemm_f16a(workspace, a_ts, b_codes, b_scales, b_ts, M, N, K, C, ldc,
+                                  static_cast<uint8_t*>(workspace) + M * K * 2, workspace_bytes - M * K * 2, status_word,
+                                  s);
+  } else {
+    st = mixfp4::launch_gemm(a_codes, a_scales, a_ts, b_codes, b_scales, b_ts, M, N, K, C, ldc, status_word, s);
+  }
   if (st) return st;
   return launch_status();
+}
+
+}  // namespace
+
+int mixfp4_gemm_workspace(int64_t M, int64_t N, int64_t K, int64_t* bytes) {
+  if (!bytes) return MIXFP4_ERR_NULL;
+  if (M < 0 || N < 0 || K < 0 || K % 256 != 0) return MIXFP4_ERR_SHAPE;
+  *bytes = gemm_scratch(M, N, K);
+  return MIXFP4_OK;
+}
+
+int mixfp4_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts,
+                const uint8_t* b_codes, const uint8_t* b_scales, const float* b_ts,
+                int64_t M, int64_t N, int64_t K, float* C, int64_t ldc,
+                uint32_t* status_word, void* stream) {
+  return gemm_impl(a_codes, a_scales, a_ts, b_codes, b_scales, b_ts, M, N, K, C, ldc, nullptr, 0, status_word, stream);
+}
+
+int mixfp4_gemm_ws(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts,
+                   const uint8_t* b_codes, const uint8_t* b_scales, const float* b_ts,
+                   int64_t M, int64_t N, int64_t K, float* C, int64_t ldc, void* workspace, int64_t workspace_bytes,
+                   uint32_t* status_word, void* stream) {
+  return gemm_impl(a_codes, a_scales, a_ts, b_codes, b_scales, b_ts, M, N, K, C, ldc, workspace, workspace_bytes,
+                   status_word, stream);
+}
+
+int mixfp4_linear_workspace(int64_t M, int64_t N, int64_t K, int64_t* bytes) {
+  if (!bytes) return MIXFP4_ERR_NULL;
+  if (M < 0 || N < 0 || K < 0 || K % 256 != 0) return MIXFP4_ERR_SHAPE;
+  if (M > (1 << 30) || N > (1 << 30) || K > (1 << 30)) return MIXFP4_ERR_SHAPE;
+  *bytes = 2 * M * K + 512;
+  if (M > 64 && N > 0 && K > 0) *bytes += mixfp4::gemm_f16a_parts_bytes(M, N, K);
+  return MIXFP4_OK;
 }
 
 int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, int mode, const uint8_t* w_codes,
@@ -331,14 +383,35 @@ int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, i
   if (!workspace) return MIXFP4_ERR_NULL;
   if (!aligned(workspace, 256)) return MIXFP4_ERR_ALIGN;
   if (M > (1 << 30) || N > (1 << 30) || K > (1 << 30) || workspace_bytes < 2 * M * K + 512) return MIXFP4_ERR_SHAPE;
-  // Scratch: the amax word and s32, then the codes, then the block scales.
+  // Scratch: the amax word and s32, then the quantized activations: decoded to
+  // f16 for the GEMM that takes A so, as codes and block scales for few rows.
   uint32_t* amax_word = static_cast<uint32_t*>(workspace);
   float* x_ts = static_cast<float*>(workspace) + 4;
-  uint8_t* codes = static_cast<uint8_t*>(workspace) + 256;
-  uint8_t* scales = codes + M * (K / 2);  // K / 2 is a multiple of 128
-  if (int st = mixfp4_quantize(x, dtype, M, K, ldx, codes, scales, x_ts, amax_word, mode, MIXFP4_SCALE_COMPUTE, stream))
+  uint8_t* xq = static_cast<uint8_t*>(workspace) + 256;
+  if (M <= 64) {
+    uint8_t* x_scales = xq + M * (K / 2);  // K / 2 is a multiple of 128
+    if (int st = mixfp4_quantize(x, dtype, M, K, ldx, xq, x_scales, x_ts, amax_word, mode, MIXFP4_SCALE_COMPUTE, stream))
+      return st;
+    return mixfp4_gemm(xq, x_scales, x_ts, w_codes, w_scales, w_ts, M, N, K, C, ldc, status_word, stream);
+  }
+  if (dtype != MIXFP4_DTYPE_BF16) return MIXFP4_ERR_DTYPE;
+  if (mode < MIXFP4_MODE_MIX || mode > MIXFP4_MODE_FOUR_SIX) return MIXFP4_ERR_ARG;
+  if (!x || !w_codes || !w_scales || !w_ts || !C) return MIXFP4_ERR_NULL;
+  if (!aligned(x, 32) || ldx % 16 != 0 || !aligned(w_codes, 16) || !aligned(w_scales, 16) || !aligned(w_ts, 4) ||
+      !aligned(C, 4) || (status_word && !aligned(status_word, 4)))
+    return MIXFP4_ERR_ALIGN;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (status_word && cudaMemsetAsync(status_word, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
+  const uint16_t* xb = static_cast<const uint16_t*>(x);
+  if (cudaMemsetAsync(amax_word, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
+  mixfp4::launch_amax(xb, M, K, ldx, amax_word, s);
+  if (int st = launch_status()) return st;
+  mixfp4::launch_quantize_f16(xb, M, K, ldx, xq, x_ts, amax_word, mode, s);
+  if (int st = launch_status()) return st;
+  if (int st = mixfp4::launch_gemm_f16a(xq, x_ts, w_codes, w_scales, w_ts, M, N, K, C, ldc, xq + M * K * 2,
+                                        workspace_bytes - M * K * 2 - 256, status_word, s))
     return st;
-  return mixfp4_gemm(codes, scales, x_ts, w_codes, w_scales, w_ts, M, N, K, C, ldc, status_word, stream);
+  return launch_status();
 }
 
 int mixfp4_gemm_native_fewrows(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts,

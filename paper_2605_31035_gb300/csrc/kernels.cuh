@@ -13,6 +13,8 @@ int launch_amax(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint32_
 int launch_quantize(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* codes,
                     uint8_t* scales, float* tensor_scale, const uint32_t* amax_word, int mode,
                     int scale_given, cudaStream_t stream);
+int launch_quantize_f16(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, void* out, float* tensor_scale,
+                        const uint32_t* amax_word, int mode, cudaStream_t stream);
 int launch_rht_amax(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, const uint8_t* signs,
                     uint32_t* amax_word, cudaStream_t stream);
 int launch_rht_quantize(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, const uint8_t* signs,
@@ -46,6 +48,13 @@ int launch_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_
                 const uint8_t* b_codes, const uint8_t* b_scales, const float* b_ts,
                 int64_t M, int64_t N, int64_t K, float* C, int64_t ldc, uint32_t* status_word,
                 cudaStream_t stream);
+int launch_decode_f16(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K, void* out,
+                      cudaStream_t stream);
+bool gemm_predecode_pays(int64_t M, int64_t N, int64_t K);
+int launch_gemm_f16a(const void* a_f16, const float* a_ts, const uint8_t* b_codes, const uint8_t* b_scales,
+                     const float* b_ts, int64_t M, int64_t N, int64_t K, float* C, int64_t ldc, void* parts,
+                     int64_t parts_room, uint32_t* status_word, cudaStream_t stream);
+int64_t gemm_f16a_parts_bytes(int64_t M, int64_t N, int64_t K);
 int launch_gemm_native_fewrows(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts,
                                const uint8_t* b_codes, const uint8_t* b_scales, const float* b_ts, int64_t M,
                                int64_t N, int64_t K, float* C, int64_t ldc, uint32_t* status_word,

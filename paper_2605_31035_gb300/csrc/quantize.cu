@@ -32,6 +32,7 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 
+#include "decode.cuh"
 #include "host_util.cuh"
 #include "kernels.cuh"
 #include "ptx.cuh"
@@ -41,12 +42,32 @@ namespace mixfp4 {
 
 namespace {
 
+// Where a quantized block goes: its 8 code bytes and scale byte, or (kF16) the
+// 16 decoded f16 values u * s8 of the GEMM that takes a decoded operand.
+template <bool kF16>
+__device__ __forceinline__ void store_block(uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, int64_t b,
+                                            uint32_t lo, uint32_t hi, uint32_t sb) {
+  if (kF16) {
+    const uint32_t h = cvt_f16x2_from_e4m3x2((uint16_t)(sb & 0x7Fu));
+    const uint32_t s2 = prmt(h, 0u, 0x1010u);
+    const bool e1m2 = (sb & 0x80u) != 0;
+    const uint32_t lut_lo = e1m2 ? kLutE1M2Lo : kLutE2M1Lo, lut_hi = e1m2 ? kLutE1M2Hi : kLutE2M1Hi;
+    uint32_t o[8];
+    decode8(lo, lut_lo, lut_hi, s2, o);
+    decode8(hi, lut_lo, lut_hi, s2, o + 4);
+    stg256(codes + b * 32, o);
+  } else {
+    stg64(codes + b * 8, lo, hi);
+    scales[b] = (uint8_t)sb;
+  }
+}
+
 // Persistent grid: each thread walks blocks b, b + nthr, b + 2 nthr, ... two
 // at a time (a, b): both blocks of a pair are quantized before either is
 // stored, so their independent dependency chains interleave, and the loads of
 // the next pair are in flight meanwhile.  The division method is fixed per
 // launch, so each method gets its own copy of the loop.
-template <int kMode, bool kContig, bool kScaled, bool kMarkstein>
+template <int kMode, bool kContig, bool kF16, bool kScaled, bool kMarkstein>
 __device__ __forceinline__ void quantize_pairs(const uint16_t* __restrict__ x, int64_t b, int64_t nthr,
                                                int64_t nblocks, int64_t kblocks, int64_t ldx,
                                                uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
@@ -57,19 +78,17 @@ __device__ __forceinline__ void quantize_pairs(const uint16_t* __restrict__ x, i
     uint32_t lo0, hi0, sb0, lo1, hi1, sb1;
     quantize_block<kMode, kScaled, kMarkstein>(wa, tc, tab, lo0, hi0, sb0);
     quantize_block<kMode, kScaled, kMarkstein>(wb, tc, tab, lo1, hi1, sb1);  // wb past the end: unused
-    stg64(codes + b * 8, lo0, hi0);
-    scales[b] = (uint8_t)sb0;
+    store_block<kF16>(codes, scales, b, lo0, hi0, sb0);
     if (b + 2 * nthr < nblocks) ldg256_stream(block_src<kContig>(x, b + 2 * nthr, kblocks, ldx), wa);
     if (b1 < nblocks) {
-      stg64(codes + b1 * 8, lo1, hi1);
-      scales[b1] = (uint8_t)sb1;
+      store_block<kF16>(codes, scales, b1, lo1, hi1, sb1);
       if (b1 + 2 * nthr < nblocks) ldg256_stream(block_src<kContig>(x, b1 + 2 * nthr, kblocks, ldx), wb);
     }
   }
 }
 
 // The first loads are issued before any set-up work.
-template <int kMode, bool kContig>
+template <int kMode, bool kContig, bool kF16>
 __global__ void __launch_bounds__(kQuantThreads, 4)
 quantize_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, int64_t ldx,
                 uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, float* tensor_scale,
@@ -92,11 +111,11 @@ quantize_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks
   const TensorConsts tc = tensor_consts(tensor_scale, amax_word, scale_given);
   const bool markstein = markstein_needed(tc);
   if (tc.scaled)
-    quantize_pairs<kMode, kContig, true, true>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
+    quantize_pairs<kMode, kContig, kF16, true, true>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
   else if (markstein)
-    quantize_pairs<kMode, kContig, false, true>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
+    quantize_pairs<kMode, kContig, kF16, false, true>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
   else
-    quantize_pairs<kMode, kContig, false, false>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
+    quantize_pairs<kMode, kContig, kF16, false, false>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
 }
 
 // Rotation + Algorithm 1, two blocks per thread side by side (as in
@@ -280,26 +299,29 @@ int launch_amax(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint32_
   return 0;
 }
 
-int launch_quantize(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* codes,
-                    uint8_t* scales, float* tensor_scale, const uint32_t* amax_word, int mode,
-                    int scale_given, cudaStream_t stream) {
+namespace {
+
+template <bool kF16>
+void launch_quantize_to(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* codes, uint8_t* scales,
+                        float* tensor_scale, const uint32_t* amax_word, int mode, int scale_given,
+                        cudaStream_t stream) {
   const int64_t kblocks = K / 16, nblocks = rows * kblocks;
   // Persistent grid: 4 CTAs per SM of the device, fewer for small tensors
   // (each thread takes at least two blocks).
   int64_t grid = (nblocks + 2 * kQuantThreads - 1) / (2 * kQuantThreads);
   if (grid > num_sms() * 4) grid = num_sms() * 4;
-  if (grid == 0) return 0;
+  if (grid == 0) return;
   // Launched as a programmatic dependent: it overlaps its launch with the tail
   // of the kernel before it (see the waits at the top of quantize_kernel).
   const int after_amax = !scale_given;
-#define MIXFP4_LAUNCH_Q(MODE)                                                                           \
-  do {                                                                                                  \
-    if (ldx == K)                                                                                       \
-      launch_pdl(quantize_kernel<MODE, true>, (unsigned)grid, kQuantThreads, 0, stream, x, nblocks,      \
-                 kblocks, ldx, codes, scales, tensor_scale, amax_word, scale_given, after_amax);        \
-    else                                                                                                \
-      launch_pdl(quantize_kernel<MODE, false>, (unsigned)grid, kQuantThreads, 0, stream, x, nblocks,     \
-                 kblocks, ldx, codes, scales, tensor_scale, amax_word, scale_given, after_amax);        \
+#define MIXFP4_LAUNCH_Q(MODE)                                                                             \
+  do {                                                                                                    \
+    if (ldx == K)                                                                                         \
+      launch_pdl(quantize_kernel<MODE, true, kF16>, (unsigned)grid, kQuantThreads, 0, stream, x, nblocks,  \
+                 kblocks, ldx, codes, scales, tensor_scale, amax_word, scale_given, after_amax);          \
+    else                                                                                                  \
+      launch_pdl(quantize_kernel<MODE, false, kF16>, (unsigned)grid, kQuantThreads, 0, stream, x, nblocks, \
+                 kblocks, ldx, codes, scales, tensor_scale, amax_word, scale_given, after_amax);          \
   } while (0)
   switch (mode) {
     case MIXFP4_MODE_MIX: MIXFP4_LAUNCH_Q(MIXFP4_MODE_MIX); break;
@@ -308,6 +330,22 @@ int launch_quantize(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uin
     default: MIXFP4_LAUNCH_Q(MIXFP4_MODE_E1M2_ONLY); break;
   }
 #undef MIXFP4_LAUNCH_Q
+}
+
+}  // namespace
+
+int launch_quantize(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* codes,
+                    uint8_t* scales, float* tensor_scale, const uint32_t* amax_word, int mode,
+                    int scale_given, cudaStream_t stream) {
+  launch_quantize_to<false>(x, rows, K, ldx, codes, scales, tensor_scale, amax_word, mode, scale_given, stream);
+  return 0;
+}
+
+// The quantized tensor as f16 values u * s8, [rows][K] (the operand of launch_gemm_f16a).
+int launch_quantize_f16(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, void* out, float* tensor_scale,
+                        const uint32_t* amax_word, int mode, cudaStream_t stream) {
+  launch_quantize_to<true>(x, rows, K, ldx, static_cast<uint8_t*>(out), nullptr, tensor_scale, amax_word, mode, 0,
+                           stream);
   return 0;
 }
 

@@ -63,8 +63,14 @@ def lib() -> ctypes.CDLL:
         L.mixfp4_dequantize.argtypes = [P, P, P, I64, I64, P, P]
         L.mixfp4_gemm.restype = I
         L.mixfp4_gemm.argtypes = [P, P, P, P, P, P, I64, I64, I64, P, I64, P, P]
+        L.mixfp4_linear_workspace.restype = I
+        L.mixfp4_linear_workspace.argtypes = [I64, I64, I64, ctypes.POINTER(I64)]
         L.mixfp4_linear.restype = I
         L.mixfp4_linear.argtypes = [P, I, I64, I64, I64, I, P, P, P, I64, P, I64, P, I64, P, P]
+        L.mixfp4_gemm_ws.restype = I
+        L.mixfp4_gemm_ws.argtypes = [P, P, P, P, P, P, I64, I64, I64, P, I64, P, I64, P, P]
+        L.mixfp4_gemm_workspace.restype = I
+        L.mixfp4_gemm_workspace.argtypes = [I64, I64, I64, ctypes.POINTER(I64)]
         L.mixfp4_split_native.restype = I
         L.mixfp4_split_native.argtypes = [P, P, I64, I64, P, P, P, P]
         L.mixfp4_gemm_native.restype = I
@@ -401,6 +407,11 @@ def _gemm_out(out, M: int, N: int, device):
         return torch.empty(M, N, dtype=torch.float32, device=device)
     _check_c(out, M, N, device)
     return out
+def gemm_workspace_bytes(M: int, N: int, K: int) -> int:
+    """Bytes of scratch memory mixfp4_gemm_ws takes for an M x N x K product (0: none)."""
+    n = ctypes.c_int64(0)
+    _check("mixfp4_gemm", lib().mixfp4_gemm_workspace(M, N, K, ctypes.byref(n)))
+    return n.value
 
 
 def mixfp4_gemm(a: QTensor, b: QTensor, out: torch.Tensor | None = None,
@@ -412,9 +423,14 @@ def mixfp4_gemm(a: QTensor, b: QTensor, out: torch.Tensor | None = None,
     M, N, K = a.rows, b.rows, a.K
     C = _gemm_out(out, M, N, a.codes.device)
     _check_status(status_word, a.codes.device)
-    st = lib().mixfp4_gemm(_ptr(a.codes), _ptr(a.scales), _ptr(a.tensor_scale),
-                           _ptr(b.codes), _ptr(b.scales), _ptr(b.tensor_scale),
-                           M, N, K, _ptr(C), C.stride(0), _ptr(status_word), _stream(stream))
+    ws_bytes = gemm_workspace_bytes(M, N, K) if K % 256 == 0 else 0
+    ws = _scratch(ws_bytes, a.codes.device) if ws_bytes > 0 else None
+    st = lib().mixfp4_gemm_ws(_ptr(a.codes), _ptr(a.scales), _ptr(a.tensor_scale),
+                              _ptr(b.codes), _ptr(b.scales), _ptr(b.tensor_scale),
+                              M, N, K, _ptr(C), C.stride(0), _ptr(ws), ws_bytes, _ptr(status_word),
+                              _stream(stream))
+    if ws is not None and stream is not None:
+        ws.record_stream(stream)  # allocated on the current stream, used on the caller's
     _check("mixfp4_gemm", st)
     return C
 
@@ -550,11 +566,14 @@ def linear(x: torch.Tensor, w_q: QTensor, mode: int = MODE_MIX, stream=None) -> 
         _check_operand(w_q, "b")
         N = w_q.codes.shape[0]
         C = torch.empty(M, N, dtype=torch.float32, device=x.device)
-        ws = _scratch(2 * M * K + 512, x.device)
+        # One scratch buffer for the quantized activations (and the parts of a split K).
+        n = ctypes.c_int64(0)
+        L = lib()
+        ws = _scratch(n.value, x.device) if L.mixfp4_linear_workspace(M, N, K, ctypes.byref(n)) == 0 else None
         if ws is not None:
-            st = lib().mixfp4_linear(_ptr(x), DTYPE_BF16, M, K, x.stride(0), int(mode), _ptr(w_q.codes),
-                                     _ptr(w_q.scales), _ptr(w_q.tensor_scale), N, _ptr(C), N, _ptr(ws), ws.numel(),
-                                     None, _stream(stream))
+            st = L.mixfp4_linear(_ptr(x), DTYPE_BF16, M, K, x.stride(0), int(mode), _ptr(w_q.codes),
+                                 _ptr(w_q.scales), _ptr(w_q.tensor_scale), N, _ptr(C), N, _ptr(ws), ws.numel(),
+                                 None, _stream(stream))
             if stream is not None:
                 ws.record_stream(stream)  # allocated on the current stream, used on the caller's
             if st in (0, _ERR_CUDA):

@@ -1,0 +1,84 @@
+"""The GEMM with A decoded to f16 beforehand (mixfp4_gemm_ws): every edge of
+its tiles and of its K split against the float64 product of the dequantized
+operands, within the 1e-5 |A| |B| bound of every GEMM path, and equal
+dispatch results without a workspace."""
+import ctypes
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+def operands(M, N, K, seed):
+    from paper_2605_31035_gb300 import ops, synth
+    x = synth.activations(M, K, seed, seed + 1).to(DEV)
+    w = synth.weights(N, K, seed + 2, 0.02, 0.5).to(DEV)
+    return ops.mixfp4_quantize(x), ops.mixfp4_quantize(w)
+
+
+def reference(a, b):
+    from paper_2605_31035_gb300 import ops
+    A, B = ops.mixfp4_dequantize(a).double(), ops.mixfp4_dequantize(b).double()
+    # The fp32 dequantization rounds v s8 s32 once per element: 2^-24 relative
+    # on each factor, 1.2e-7 of |A| |B| in all, inside the 1e-5 bound.
+    return A @ B.T, A.abs() @ B.abs().T
+
+
+def call(a, b, C, ws):
+    from paper_2605_31035_gb300 import ops
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    p = ops._ptr
+    st = ops.lib().mixfp4_gemm_ws(p(a.codes), p(a.scales), p(a.tensor_scale), p(b.codes), p(b.scales),
+                                  p(b.tensor_scale), a.rows, b.rows, a.K, p(C), C.stride(0), p(ws),
+                                  0 if ws is None else ws.numel(), p(status),
+                                  ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == 0
+    torch.cuda.synchronize()
+    assert status.item() == 0
+
+
+# Sizes at which the decode pass is taken: one row and one column past a tile,
+# the narrowest tiles, several waves, K split over all pairs (few tiles, long
+# K), K over several accumulation chunks, N not a multiple of 4 (C row stride
+# without 16-byte alignment).
+@pytest.mark.parametrize("M,N,K", [(65, 96, 2304), (256, 97, 2560), (257, 300, 2304), (129, 33, 4352),
+                                   (100, 512, 14336), (300, 1000, 8192), (777, 3000, 2816), (513, 4101, 2560),
+                                   (2050, 4100, 2304), (700, 301, 8448)])
+def test_decoded_a_within_bound(M, N, K):
+    from paper_2605_31035_gb300 import ops
+    a, b = operands(M, N, K, 8100 + M)
+    need = ops.gemm_workspace_bytes(M, N, K)
+    assert need >= 2 * M * K
+    C = torch.full((M, N), float("nan"), device=DEV)
+    call(a, b, C, torch.empty(need, dtype=torch.uint8, device=DEV))
+    ref, D = reference(a, b)
+    assert torch.all((C.double() - ref).abs() <= 1e-5 * D)
+    C2 = torch.full((M, N), float("nan"), device=DEV)
+    call(a, b, C2, None)                       # no workspace: A decoded in the main loop
+    assert torch.all((C2.double() - ref).abs() <= 1e-5 * D)
+
+
+def test_strided_and_unaligned_output():
+    """C inside a wider buffer, whose base and row stride are 4-byte aligned
+    only: the columns around it stay untouched."""
+    from paper_2605_31035_gb300 import ops
+    M, N, K = 300, 500, 2560
+    a, b = operands(M, N, K, 8500)
+    ws = torch.empty(ops.gemm_workspace_bytes(M, N, K), dtype=torch.uint8, device=DEV)
+    ref, D = reference(a, b)
+    for width, off in ((512, 8), (507, 3)):
+        big = torch.full((M, width), -3.0, device=DEV)
+        call(a, b, big[:, off:off + N], ws)
+        assert torch.all((big[:, off:off + N].double() - ref).abs() <= 1e-5 * D)
+        assert torch.all(big[:, :off] == -3.0) and torch.all(big[:, off + N:] == -3.0)
+
+
+def test_small_products_take_no_workspace():
+    from paper_2605_31035_gb300 import ops
+    need = ops.gemm_workspace_bytes
+    assert need(64, 4096, 4096) == 0          # the few-row path
+    assert need(8000, 300, 8192) == 0         # one tile column: nothing to save
+    assert need(0, 4096, 4096) == 0 and need(100, 0, 4096) == 0
