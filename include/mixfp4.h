@@ -319,12 +319,15 @@ int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, i
 int mixfp4_linear_workspace(int64_t M, int64_t N, int64_t K, int64_t* bytes);
 
 /*
- * mixfp4_gemm_ws -- mixfp4_gemm with scratch memory.  With `workspace_bytes`
- * >= the bytes mixfp4_gemm_workspace reports (and those positive) A is first decoded
- * to f16 in the workspace (App. B.5 values times the block scales, exact), so
- * the main loop decodes only B, and a long K may be cut into parts that run
- * side by side (their sum is compensated); otherwise, and with workspace = NULL, the call
- * is mixfp4_gemm.
+ * mixfp4_gemm_ws -- mixfp4_gemm with scratch memory, for the same result
+ * (App. B.1 Eq. (factor)).  With `workspace_bytes` >= the bytes
+ * mixfp4_gemm_workspace reports (and those positive):
+ *   M > 64   A is first decoded to f16 in the workspace (App. B.5 values times
+ *            the block scales, exact), so the main loop decodes only B;
+ *   M <= 64  the codes themselves are contracted on the block-scaled FP4 tensor
+ *            path (exact products, as in mixfp4_gemm_native_fewrows);
+ * and K may be cut into parts that run side by side (their sum is compensated).
+ * Otherwise, and with workspace = NULL, the call is mixfp4_gemm.
  *
  * workspace       device, 256-byte aligned, or NULL; written by the call and free
  *                 for reuse once the call's work on `stream` is done.

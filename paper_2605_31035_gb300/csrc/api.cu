@@ -296,10 +296,15 @@ namespace {
 // Workspace of mixfp4_gemm_ws: A decoded to f16 where that pays (2 M K bytes, a
 // multiple of 512), then the parts of a split K.
 int64_t gemm_scratch(int64_t M, int64_t N, int64_t K) {
-  if (M <= 64 || N <= 0 || K <= 0 || M > (1 << 30) || N > (1 << 30) || K > (1 << 30)) return 0;
+  if (M <= 0 || N <= 0 || K <= 0 || M > (1 << 30) || N > (1 << 30) || K > (1 << 30)) return 0;
+  if (M <= 64) return mixfp4::fewrows_scratch_bytes(M, N, K);
   if (!mixfp4::gemm_predecode_pays(M, N, K)) return 0;
   return M * K * 2 + mixfp4::gemm_f16a_parts_bytes(M, N, K);
 }
+
+// mixfp4_linear's scratch for up to 64 rows: amax word and s32 (256 bytes), the
+// codes, the block scales, then (at the returned offset) launch_fewrows' own.
+int64_t few_rows_offset(int64_t M, int64_t K) { return (256 + M * (K / 2) + M * (K / 16) + 255) / 256 * 256; }
 
 // Shared body of the decode-path GEMM entry points.
 int gemm_impl(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts, const uint8_t* b_codes,
@@ -327,6 +332,9 @@ int gemm_impl(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts
   int st;
   if (need > 0 && workspace && workspace_bytes >= need) {
     if (!aligned(workspace, 256)) return MIXFP4_ERR_ALIGN;
+    if (M <= 64)
+      return mixfp4::launch_fewrows(a_codes, a_scales, a_ts, b_codes, b_scales, b_ts, M, N, K, C, ldc, workspace,
+                                    status_word, s);
     if (mixfp4::launch_decode_f16(a_codes, a_scales, M, K, workspace, s) != 0) return MIXFP4_ERR_CUDA;
     st = mixfp4::launch_gemm_f16a(workspace, a_ts, b_codes, b_scales, b_ts, M, N, K, C, ldc,
                                   static_cast<uint8_t*>(workspace) + M * K * 2, workspace_bytes - M * K * 2, status_word,
@@ -367,7 +375,13 @@ int mixfp4_linear_workspace(int64_t M, int64_t N, int64_t K, int64_t* bytes) {
   if (M < 0 || N < 0 || K < 0 || K % 256 != 0) return MIXFP4_ERR_SHAPE;
   if (M > (1 << 30) || N > (1 << 30) || K > (1 << 30)) return MIXFP4_ERR_SHAPE;
   *bytes = 2 * M * K + 512;
-  if (M > 64 && N > 0 && K > 0) *bytes += mixfp4::gemm_f16a_parts_bytes(M, N, K);
+  if (M == 0 || N == 0 || K == 0) return MIXFP4_OK;
+  if (M > 64) {
+    *bytes += mixfp4::gemm_f16a_parts_bytes(M, N, K);
+  } else {
+    const int64_t few = few_rows_offset(M, K) + mixfp4::fewrows_scratch_bytes(M, N, K);
+    if (few > *bytes) *bytes = few;
+  }
   return MIXFP4_OK;
 }
 
@@ -392,7 +406,9 @@ int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, i
     uint8_t* x_scales = xq + M * (K / 2);  // K / 2 is a multiple of 128
     if (int st = mixfp4_quantize(x, dtype, M, K, ldx, xq, x_scales, x_ts, amax_word, mode, MIXFP4_SCALE_COMPUTE, stream))
       return st;
-    return mixfp4_gemm(xq, x_scales, x_ts, w_codes, w_scales, w_ts, M, N, K, C, ldc, status_word, stream);
+    const int64_t off = few_rows_offset(M, K);
+    return mixfp4_gemm_ws(xq, x_scales, x_ts, w_codes, w_scales, w_ts, M, N, K, C, ldc,
+                          static_cast<uint8_t*>(workspace) + off, workspace_bytes - off, status_word, stream);
   }
   if (dtype != MIXFP4_DTYPE_BF16) return MIXFP4_ERR_DTYPE;
   if (mode < MIXFP4_MODE_MIX || mode > MIXFP4_MODE_FOUR_SIX) return MIXFP4_ERR_ARG;

@@ -459,33 +459,29 @@ gemm_f16a_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   }
 }
 
-// C = s32A s32B / 4 x the sum of the parts of a split K (parts of m_pad x ldp
-// floats), four columns per thread.  The sum carries its rounding errors along
+// C = factor x s32A x s32B x the sum of the parts of a split product (part_stride
+// floats apart, rows of ldp floats), four columns per thread.  The sum carries its rounding errors along
 // (Knuth's two-sum), so splitting K costs no accuracy: on 100 x 512 x 14336 the
 // parts added into C one by one in fp32 left twice the error of one pass.
 __global__ void __launch_bounds__(256)
 sum_parts_kernel(const float* __restrict__ parts, int splits, long long part_stride, int ldp,
-                 const float* __restrict__ a_ts, const float* __restrict__ b_ts, int M, int N, float* __restrict__ C,
-                 long long ldc, int vec) {
+                 float factor, const float* __restrict__ a_ts, const float* __restrict__ b_ts, int M, int N,
+                 float* __restrict__ C, long long ldc, int vec) {
   griddep_wait();
   griddep_launch_dependents();
-  const float sa = 0.25f * __ldg(a_ts), sb = __ldg(b_ts);
+  const float sa = factor * __ldg(a_ts), sb = __ldg(b_ts);  // factor: a power of two
   const int q_n = (N + 3) / 4;
   const long long n = (long long)M * q_n;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const int m = (int)(i / q_n), c = (int)(i - (long long)m * q_n) * 4;
     const float* p = parts + (long long)m * ldp + c;
     float s[4] = {0.0f, 0.0f, 0.0f, 0.0f}, e[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll 4
+#pragma unroll 8
     for (int j = 0; j < splits; ++j) {
       const float4 v4 = __ldg(reinterpret_cast<const float4*>(p + j * part_stride));
       const float v[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float t = __fadd_rn(s[k], v[k]), z = __fsub_rn(t, s[k]);
-        e[k] = __fadd_rn(e[k], __fadd_rn(__fsub_rn(s[k], __fsub_rn(t, z)), __fsub_rn(v[k], z)));
-        s[k] = t;
-      }
+      for (int k = 0; k < 4; ++k) two_sum_add(s[k], e[k], v[k]);
     }
     float o[4];
 #pragma unroll
@@ -585,6 +581,17 @@ int64_t gemm_f16a_parts_bytes(int64_t M, int64_t N, int64_t K) {
   return parts_bytes(M, N, make_plan(M, N, K, INT64_MAX).splits);
 }
 
+int launch_sum_parts(const float* parts, int splits, int64_t part_stride, int64_t ldp, float factor, const float* a_ts,
+                     const float* b_ts, int64_t M, int64_t N, float* C, int64_t ldc, cudaStream_t stream) {
+  const int vec = ((ldc & 3) == 0) && ((reinterpret_cast<uintptr_t>(C) & 15) == 0);
+  int64_t grid = (M * ((N + 3) / 4) + 255) / 256;
+  if (grid > num_sms() * 8) grid = num_sms() * 8;
+  return launch_pdl(fa::sum_parts_kernel, (unsigned)grid, 256, 0, stream, parts, splits, (long long)part_stride,
+                    (int)ldp, factor, a_ts, b_ts, (int)M, (int)N, C, (long long)ldc, vec) == cudaSuccess
+             ? MIXFP4_OK
+             : MIXFP4_ERR_CUDA;
+}
+
 int launch_gemm_f16a(const void* a_f16, const float* a_ts, const uint8_t* b_codes, const uint8_t* b_scales,
                      const float* b_ts, int64_t M, int64_t N, int64_t K, float* C, int64_t ldc, void* parts,
                      int64_t parts_room, uint32_t* status_word, cudaStream_t stream) {
@@ -631,14 +638,9 @@ int launch_gemm_f16a(const void* a_f16, const float* a_ts, const uint8_t* b_code
                  tmc, c_tma, a_ts, b_ts, (int)M, (int)N, (int)K, C, (long long)ldc, p.tile_n, (int)p.dp_tiles,
                  kAccumChunkK / fa::BKC, p.splits, p.kps, status_word) != cudaSuccess)
     return MIXFP4_ERR_CUDA;
-  if (p.splits > 1) {
-    int64_t grid = (M * ((N + 3) / 4) + 255) / 256;
-    if (grid > num_sms() * 8) grid = num_sms() * 8;
-    if (launch_pdl(fa::sum_parts_kernel, (unsigned)grid, 256, 0, stream, static_cast<const float*>(parts), p.splits,
-                   (long long)(m_pad * ldp), (int)ldp, a_ts, b_ts, (int)M, (int)N, C, (long long)ldc, c_vec) !=
-        cudaSuccess)
-      return MIXFP4_ERR_CUDA;
-  }
+  if (p.splits > 1)
+    return launch_sum_parts(static_cast<const float*>(parts), p.splits, m_pad * ldp, ldp, 0.25f, a_ts, b_ts, M, N, C,
+                            ldc, stream);
   return MIXFP4_OK;
 }
 

@@ -55,6 +55,12 @@ int launch_gemm_f16a(const void* a_f16, const float* a_ts, const uint8_t* b_code
                      const float* b_ts, int64_t M, int64_t N, int64_t K, float* C, int64_t ldc, void* parts,
                      int64_t parts_room, uint32_t* status_word, cudaStream_t stream);
 int64_t gemm_f16a_parts_bytes(int64_t M, int64_t N, int64_t K);
+int launch_sum_parts(const float* parts, int splits, int64_t part_stride, int64_t ldp, float factor, const float* a_ts,
+                     const float* b_ts, int64_t M, int64_t N, float* C, int64_t ldc, cudaStream_t stream);
+int64_t fewrows_scratch_bytes(int64_t M, int64_t N, int64_t K);
+int launch_fewrows(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts, const uint8_t* b_codes,
+                   const uint8_t* b_scales, const float* b_ts, int64_t M, int64_t N, int64_t K, float* C, int64_t ldc,
+                   void* scratch, uint32_t* status_word, cudaStream_t stream);
 int launch_gemm_native_fewrows(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts,
                                const uint8_t* b_codes, const uint8_t* b_scales, const float* b_ts, int64_t M,
                                int64_t N, int64_t K, float* C, int64_t ldc, uint32_t* status_word,

@@ -50,6 +50,7 @@
 #include "kernels.cuh"
 #include "pipeline.cuh"
 #include "ptx.cuh"
+#include "residual.cuh"
 #include "sm100.cuh"
 
 namespace mixfp4 {
@@ -64,7 +65,6 @@ using namespace sm100;
 // payload 2 where p0 p2 (p = 5, 7); both keep the sign bit.  Each line is one
 // three-input logic instruction (lop3; truth-table byte from a = 0xF0,
 // b = 0xCC, c = 0xAA).
-#define MIXFP4_LOP3(d, a, b, c, LUT) asm("lop3.b32 %0, %1, %2, %3, " #LUT ";" : "=r"(d) : "r"(a), "r"(b), "r"(c))
 __device__ __forceinline__ void split_e1m2_word(uint32_t w, uint32_t tmask, uint32_t& main, uint32_t& res) {
   const uint32_t r1 = w >> 1, r2 = w >> 2, l1 = w << 1;
   uint32_t m0, m1, t, r;
@@ -553,19 +553,6 @@ struct Bars {
 };
 static_assert(sizeof(Bars) <= 256, "barrier block");
 
-// Residual E2M1 codes of eight nibbles (sign in bit 3, payload p in bits
-// 0-2): payload {0,1,2,3,4,4,4,2}[p] = p & F with F's bit 0 = ~p2, bit 1 =
-// ~p2 | p0, bit 2 = ~(p1 & p0), and the sign kept.  Checked exhaustively on
-// the host against the table.
-__device__ __forceinline__ uint32_t residual_word(uint32_t w) {
-  const uint32_t r1 = w >> 1, r2 = w >> 2, l1 = w << 1, l2 = w << 2;
-  uint32_t a, b, c, d;
-  MIXFP4_LOP3(a, 0x22222222u, r1, l1, 0xBF);        // ~K | ~r1 | l1
-  MIXFP4_LOP3(b, 0x44444444u, l1, l2, 0x7F);        // ~K | ~(l1 & l2)
-  MIXFP4_LOP3(c, w, a, b, 0x80);                    // w & a & b
-  MIXFP4_LOP3(d, c, r2, 0x11111111u, 0x70);         // c & (~r2 | ~K)
-  return d;
-}
 // Scale bytes of a residual row: the scale (type bit cleared) where the type
 // bit is set, else 0 (prmt with the sign-replicate selectors gives 0xFF per
 // byte whose bit 7 is set).

@@ -41,6 +41,14 @@ __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, 
                : "memory");
 }
 
+// s + e <- s + e + v with the rounding error of the addition kept in e (Knuth's
+// two-sum; e itself accumulates in fp32).
+__device__ __forceinline__ void two_sum_add(float& s, float& e, float v) {
+  const float t = __fadd_rn(s, v), z = __fsub_rn(t, s);
+  e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z)));
+  s = t;
+}
+
 // Work schedule of one CTA pair, walked identically by every role.  Tiles
 // below dp_tiles are whole-tile work, dealt round-robin (tile = cluster,
 // cluster + nclusters, ...).  The (tile, 256-wide K slice) units of the

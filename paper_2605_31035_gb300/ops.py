@@ -425,14 +425,17 @@ def mixfp4_gemm(a: QTensor, b: QTensor, out: torch.Tensor | None = None,
     _check_status(status_word, a.codes.device)
     ws_bytes = gemm_workspace_bytes(M, N, K) if K % 256 == 0 else 0
     ws = _scratch(ws_bytes, a.codes.device) if ws_bytes > 0 else None
-    st = lib().mixfp4_gemm_ws(_ptr(a.codes), _ptr(a.scales), _ptr(a.tensor_scale),
-                              _ptr(b.codes), _ptr(b.scales), _ptr(b.tensor_scale),
-                              M, N, K, _ptr(C), C.stride(0), _ptr(ws), ws_bytes, _ptr(status_word),
-                              _stream(stream))
+    _check("mixfp4_gemm", _gemm_ws(a, b, C, ws, status_word, stream))
+    return C
+
+
+def _gemm_ws(a: QTensor, b: QTensor, C, ws, status_word, stream) -> int:
+    st = lib().mixfp4_gemm_ws(_ptr(a.codes), _ptr(a.scales), _ptr(a.tensor_scale), _ptr(b.codes), _ptr(b.scales),
+                              _ptr(b.tensor_scale), a.rows, b.rows, a.K, _ptr(C), C.stride(0), _ptr(ws),
+                              0 if ws is None else ws.numel(), _ptr(status_word), _stream(stream))
     if ws is not None and stream is not None:
         ws.record_stream(stream)  # allocated on the current stream, used on the caller's
-    _check("mixfp4_gemm", st)
-    return C
+    return st
 
 
 @dataclass
@@ -512,8 +515,8 @@ def mixfp4_gemm_native(a: NativeTensor, b: NativeTensor, out: torch.Tensor | Non
 def mixfp4_gemm_native_fewrows(a: QTensor, b: QTensor, out: torch.Tensor | None = None,
                                status_word: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """C = A_deq . B_deq^T for a with at most 64 rows, on the block-scaled FP4
-    tensor path: the stored codes are the main E2M1 operands, their residual
-    rows and scale tiles are formed on the fly."""
+    tensor path: the stored codes are the main E2M1 operands, what their E1M2
+    blocks need beside them and the scale tiles are formed on the fly."""
     _check_operand(a, "a")
     _check_operand(b, "b")
     _require(a.K == b.K and a.rows <= 64 and a.codes.device == b.codes.device,
@@ -521,6 +524,11 @@ def mixfp4_gemm_native_fewrows(a: QTensor, b: QTensor, out: torch.Tensor | None 
     M, N, K = a.rows, b.rows, a.K
     C = _gemm_out(out, M, N, a.codes.device)
     _check_status(status_word, a.codes.device)
+    ws_bytes = gemm_workspace_bytes(M, N, K) if K % 256 == 0 else 0
+    ws = _scratch(ws_bytes, a.codes.device) if ws_bytes > 0 else None
+    if ws is not None:
+        _check("mixfp4_gemm_native_fewrows", _gemm_ws(a, b, C, ws, status_word, stream))
+        return C
     st = lib().mixfp4_gemm_native_fewrows(_ptr(a.codes), _ptr(a.scales), _ptr(a.tensor_scale),
                                           _ptr(b.codes), _ptr(b.scales), _ptr(b.tensor_scale),
                                           M, N, K, _ptr(C), C.stride(0), _ptr(status_word), _stream(stream))

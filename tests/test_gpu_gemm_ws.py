@@ -76,9 +76,45 @@ def test_strided_and_unaligned_output():
         assert torch.all(big[:, :off] == -3.0) and torch.all(big[:, off + N:] == -3.0)
 
 
+# The few-row path (M <= 64): the last row counts of its three operand widths
+# and the first beyond, one weight row, one before and after a 128-row tile, one
+# and several units of K, K in one and in many parts, every block type mix.
+@pytest.mark.parametrize("M,N,K,mode", [(1, 1, 256, 0), (16, 129, 512, 0), (17, 127, 768, 2), (32, 4096, 1280, 0),
+                                        (33, 300, 4352, 0), (64, 700, 14336, 0), (5, 20000, 1024, 1),
+                                        (64, 513, 256, 3), (2, 300, 8192, 2), (48, 28672, 512, 0)])
+def test_few_rows_within_bound(M, N, K, mode):
+    from paper_2605_31035_gb300 import ops, synth
+    a = ops.mixfp4_quantize(synth.activations(M, K, 8700 + M, 8701).to(DEV), mode)
+    b = ops.mixfp4_quantize(synth.weights(N, K, 8702 + M, 0.02, 0.5).to(DEV), mode)
+    ws = torch.empty(ops.gemm_workspace_bytes(M, N, K), dtype=torch.uint8, device=DEV)
+    ref, D = reference(a, b)
+    for width, off in ((N, 0), (N + 5, 3)):    # dense, then inside a wider buffer off 16-byte alignment
+        big = torch.full((M, width), -3.0, device=DEV)
+        call(a, b, big[:, off:off + N], ws)
+        assert torch.all((big[:, off:off + N].double() - ref).abs() <= 1e-5 * D)
+        assert torch.all(big[:, :off] == -3.0) and torch.all(big[:, off + N:] == -3.0)
+
+
+def test_few_rows_extreme_scales():
+    """Blocks whose scale is 0, the smallest subnormal and 448, in both types,
+    against every payload and sign."""
+    from paper_2605_31035_gb300 import ops
+    g = torch.Generator(device="cpu").manual_seed(5)
+    def tensor(rows, K):
+        codes = torch.randint(0, 256, (rows, K // 2), generator=g, dtype=torch.uint8)
+        pick = torch.tensor([0x00, 0x80, 0x01, 0x81, 0x07, 0x87, 0x7E, 0xFE, 0x38, 0xB8], dtype=torch.uint8)
+        scales = pick[torch.randint(0, len(pick), (rows, K // 16), generator=g)]
+        return ops.QTensor(codes.to(DEV), scales.to(DEV), torch.tensor([0.5], device=DEV))
+    a, b = tensor(20, 1024), tensor(200, 1024)
+    ws = torch.empty(ops.gemm_workspace_bytes(20, 200, 1024), dtype=torch.uint8, device=DEV)
+    C = torch.full((20, 200), float("nan"), device=DEV)
+    call(a, b, C, ws)
+    ref, D = reference(a, b)
+    assert torch.all((C.double() - ref).abs() <= 1e-5 * D)
+
+
 def test_small_products_take_no_workspace():
     from paper_2605_31035_gb300 import ops
     need = ops.gemm_workspace_bytes
-    assert need(64, 4096, 4096) == 0          # the few-row path
     assert need(8000, 300, 8192) == 0         # one tile column: nothing to save
     assert need(0, 4096, 4096) == 0 and need(100, 0, 4096) == 0
