@@ -55,6 +55,7 @@ int mixfp4_quantize(const void* x, int dtype, int64_t rows, int64_t K, int64_t l
   }
   const uint16_t* xb = static_cast<const uint16_t*>(x);
   if (!given) {
+    if (mixfp4::launch_quantize_small(xb, rows, K, ldx, codes, scales, tensor_scale, mode, s)) return launch_status();
     if (cudaMemsetAsync(workspace, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
     mixfp4::launch_amax(xb, rows, K, ldx, workspace, s);
     if (int st = launch_status()) return st;
@@ -402,14 +403,6 @@ int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, i
   uint32_t* amax_word = static_cast<uint32_t*>(workspace);
   float* x_ts = static_cast<float*>(workspace) + 4;
   uint8_t* xq = static_cast<uint8_t*>(workspace) + 256;
-  if (M <= 64) {
-    uint8_t* x_scales = xq + M * (K / 2);  // K / 2 is a multiple of 128
-    if (int st = mixfp4_quantize(x, dtype, M, K, ldx, xq, x_scales, x_ts, amax_word, mode, MIXFP4_SCALE_COMPUTE, stream))
-      return st;
-    const int64_t off = few_rows_offset(M, K);
-    return mixfp4_gemm_ws(xq, x_scales, x_ts, w_codes, w_scales, w_ts, M, N, K, C, ldc,
-                          static_cast<uint8_t*>(workspace) + off, workspace_bytes - off, status_word, stream);
-  }
   if (dtype != MIXFP4_DTYPE_BF16) return MIXFP4_ERR_DTYPE;
   if (mode < MIXFP4_MODE_MIX || mode > MIXFP4_MODE_FOUR_SIX) return MIXFP4_ERR_ARG;
   if (!x || !w_codes || !w_scales || !w_ts || !C) return MIXFP4_ERR_NULL;
@@ -419,6 +412,20 @@ int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, i
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (status_word && cudaMemsetAsync(status_word, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
   const uint16_t* xb = static_cast<const uint16_t*>(x);
+  if (M <= 64) {
+    const int64_t off = few_rows_offset(M, K), room = workspace_bytes - off;
+    uint8_t* scratch = static_cast<uint8_t*>(workspace) + off;
+    int st = 0;
+    if (room >= mixfp4::fewrows_scratch_bytes(M, N, K) &&
+        mixfp4::launch_linear_fewrows(xb, M, K, ldx, mode, x_ts, w_codes, w_scales, w_ts, N, C, ldc, scratch,
+                                      status_word, s, &st))
+      return st ? st : launch_status();
+    uint8_t* x_scales = xq + M * (K / 2);  // K / 2 is a multiple of 128
+    st = mixfp4_quantize(x, dtype, M, K, ldx, xq, x_scales, x_ts, amax_word, mode, MIXFP4_SCALE_COMPUTE, stream);
+    if (st) return st;
+    return mixfp4_gemm_ws(xq, x_scales, x_ts, w_codes, w_scales, w_ts, M, N, K, C, ldc, scratch, room, status_word,
+                          stream);
+  }
   if (cudaMemsetAsync(amax_word, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
   mixfp4::launch_amax(xb, M, K, ldx, amax_word, s);
   if (int st = launch_status()) return st;

@@ -128,9 +128,6 @@ struct Bars {
 };
 static_assert(sizeof(Bars) <= OFF_RINGS, "barrier block");
 
-// Row r's four ue4m3 scales of a K step in the tiled layout of 128 rows.
-__device__ __forceinline__ uint32_t sf_offset(int r) { return (uint32_t)((r & 31) * 16 + (r >> 5) * 4); }
-
 // Activation operand: thread = 16-byte chunk (32 codes) of one of XR rows.
 __global__ void __launch_bounds__(256)
 fewrows_prep_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales, int M, int xr, int K,
@@ -154,8 +151,8 @@ fewrows_prep_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict
   reinterpret_cast<uint4*>(xop + (int64_t)(xr + r) * (K / 2))[c] = q;
   if ((c & 1) == 0) {
     uint8_t* t = sfa + (int64_t)(c / 2) * 512;
-    *reinterpret_cast<uint32_t*>(t + sf_offset(r)) = s4 & 0x7F7F7F7Fu;
-    *reinterpret_cast<uint32_t*>(t + sf_offset(xr + r)) = s4 & 0x7F7F7F7Fu;
+    *reinterpret_cast<uint32_t*>(t + tiled_scale_row(r)) = s4 & 0x7F7F7F7Fu;
+    *reinterpret_cast<uint32_t*>(t + tiled_scale_row(xr + r)) = s4 & 0x7F7F7F7Fu;
   }
 }
 
@@ -391,7 +388,7 @@ fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
       for (int j = 0; j < 2; ++j) {  // scales of this half's two K steps, by block type
         const uint32_t sw = j ? cur.y : cur.x;
         const uint32_t t1 = sw & prmt(sw, 0u, 0xBA98u) & 0x7F7F7F7Fu;  // prmt: 0xFF bytes where the type bit is set
-        const uint32_t o = slot + (uint32_t)(2 * half + j) * 512 + sf_offset(row);
+        const uint32_t o = slot + (uint32_t)(2 * half + j) * 512 + tiled_scale_row(row);
         sts32(o, (sw & 0x7F7F7F7Fu) ^ t1);
         sts32(o + SF_UNIT, t1);
       }
@@ -490,9 +487,10 @@ int64_t fewrows_scratch_bytes(int64_t M, int64_t N, int64_t K) {
   return fr::scratch_of(M, N, K, (int)((num_kc + kps - 1) / kps)).bytes;
 }
 
-int launch_fewrows(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts, const uint8_t* b_codes,
-                   const uint8_t* b_scales, const float* b_ts, int64_t M, int64_t N, int64_t K, float* C, int64_t ldc,
-                   void* scratch, uint32_t* status_word, cudaStream_t stream) {
+// Few-row GEMM from an activation operand already in the scratch.
+static int launch_fewrows_main(const float* a_ts, const uint8_t* b_codes, const uint8_t* b_scales, const float* b_ts,
+                               int64_t M, int64_t N, int64_t K, float* C, int64_t ldc, void* scratch,
+                               uint32_t* status_word, cudaStream_t stream) {
   const int64_t num_kc = K / fr::BKC, tiles = (N + fr::WR - 1) / fr::WR;
   const int kps = fr::plan_kps(M, N, K), splits = (int)((num_kc + kps - 1) / kps), xr = fr::xr_of((int)M);
   const fr::Scratch sc = fr::scratch_of(M, N, K, splits);
@@ -505,10 +503,6 @@ int launch_fewrows(const uint8_t* a_codes, const uint8_t* a_scales, const float*
   static std::atomic<uint64_t> smem_set{0};
   if (!set_dynamic_smem_once(reinterpret_cast<const void*>(fr::fewrows_kernel), 232448, smem_set))
     return MIXFP4_ERR_CUDA;
-  const int64_t prep = xr * (K / 32);
-  if (launch_pdl(fr::fewrows_prep_kernel, (unsigned)((prep + 255) / 256), 256, 0, stream, a_codes, a_scales, (int)M, xr,
-                 (int)K, base, base + sc.sfa) != cudaSuccess)
-    return MIXFP4_ERR_CUDA;
   const int64_t items = tiles * splits;
   const int64_t grid = items < num_sms() ? items : num_sms();
   float* parts = reinterpret_cast<float*>(base + sc.parts);
@@ -518,6 +512,29 @@ int launch_fewrows(const uint8_t* a_codes, const uint8_t* a_scales, const float*
     return MIXFP4_ERR_CUDA;
   if (splits == 1) return MIXFP4_OK;
   return launch_sum_parts(parts, splits, M * tiles * fr::WR, tiles * fr::WR, 1.0f, a_ts, b_ts, M, N, C, ldc, stream);
+}
+
+int launch_fewrows(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts, const uint8_t* b_codes,
+                   const uint8_t* b_scales, const float* b_ts, int64_t M, int64_t N, int64_t K, float* C, int64_t ldc,
+                   void* scratch, uint32_t* status_word, cudaStream_t stream) {
+  const int xr = fr::xr_of((int)M);
+  uint8_t* base = static_cast<uint8_t*>(scratch);
+  const int64_t prep = xr * (K / 32);
+  if (launch_pdl(fr::fewrows_prep_kernel, (unsigned)((prep + 255) / 256), 256, 0, stream, a_codes, a_scales, (int)M, xr,
+                 (int)K, base, base + fr::scratch_of(M, N, K, 1).sfa) != cudaSuccess)
+    return MIXFP4_ERR_CUDA;
+  return launch_fewrows_main(a_ts, b_codes, b_scales, b_ts, M, N, K, C, ldc, scratch, status_word, stream);
+}
+
+bool launch_linear_fewrows(const uint16_t* x, int64_t M, int64_t K, int64_t ldx, int mode, float* x_ts,
+                           const uint8_t* w_codes, const uint8_t* w_scales, const float* w_ts, int64_t N, float* C,
+                           int64_t ldc, void* scratch, uint32_t* status_word, cudaStream_t stream, int* status) {
+  uint8_t* base = static_cast<uint8_t*>(scratch);
+  if (!launch_quantize_fewrows(x, M, K, ldx, base, base + fr::scratch_of(M, N, K, 1).sfa, x_ts, mode, fr::xr_of((int)M),
+                               stream))
+    return false;
+  *status = launch_fewrows_main(x_ts, w_codes, w_scales, w_ts, M, N, K, C, ldc, scratch, status_word, stream);
+  return true;
 }
 
 }  // namespace mixfp4

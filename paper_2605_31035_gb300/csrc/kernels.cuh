@@ -13,6 +13,10 @@ int launch_amax(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint32_
 int launch_quantize(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* codes,
                     uint8_t* scales, float* tensor_scale, const uint32_t* amax_word, int mode,
                     int scale_given, cudaStream_t stream);
+bool launch_quantize_small(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* codes, uint8_t* scales,
+                           float* tensor_scale, int mode, cudaStream_t stream);
+bool launch_quantize_fewrows(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* xop, uint8_t* sfa,
+                             float* tensor_scale, int mode, int xr, cudaStream_t stream);
 int launch_quantize_f16(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, void* out, float* tensor_scale,
                         const uint32_t* amax_word, int mode, cudaStream_t stream);
 int launch_rht_amax(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, const uint8_t* signs,
@@ -61,6 +65,11 @@ int64_t fewrows_scratch_bytes(int64_t M, int64_t N, int64_t K);
 int launch_fewrows(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts, const uint8_t* b_codes,
                    const uint8_t* b_scales, const float* b_ts, int64_t M, int64_t N, int64_t K, float* C, int64_t ldc,
                    void* scratch, uint32_t* status_word, cudaStream_t stream);
+// mixfp4_linear on few rows with the quantizer writing the GEMM's activation
+// operand: false (nothing enqueued) where the rows are too many for that.
+bool launch_linear_fewrows(const uint16_t* x, int64_t M, int64_t K, int64_t ldx, int mode, float* x_ts,
+                           const uint8_t* w_codes, const uint8_t* w_scales, const float* w_ts, int64_t N, float* C,
+                           int64_t ldc, void* scratch, uint32_t* status_word, cudaStream_t stream, int* status);
 int launch_gemm_native_fewrows(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts,
                                const uint8_t* b_codes, const uint8_t* b_scales, const float* b_ts, int64_t M,
                                int64_t N, int64_t K, float* C, int64_t ldc, uint32_t* status_word,

@@ -37,6 +37,8 @@
 #include "kernels.cuh"
 #include "ptx.cuh"
 #include "quant_core.cuh"
+#include "residual.cuh"
+#include "sm100.cuh"
 
 namespace mixfp4 {
 
@@ -116,6 +118,81 @@ quantize_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks
     quantize_pairs<kMode, kContig, kF16, false, true>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
   else
     quantize_pairs<kMode, kContig, kF16, false, false>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
+}
+
+// Small tensors in one launch: a cluster of eight CTAs holds the whole tensor in
+// registers (up to kSmallPer blocks per thread), the CTAs exchange their maxima
+// through distributed shared memory, and every thread quantizes the blocks it
+// holds.  Such a call is launches and latency, not work: memset, amax_kernel and
+// quantize_kernel took 9 us of GPU time and three launches on 16 x 8192.
+//   kOut 0: codes and block scales; 1: the activation operand of the few-row
+//   GEMM (xr main rows, xr residual rows, scales in the tiled layout), rows from
+//   `rows` to xr as zeros.
+constexpr int kSmallCtas = 8, kSmallThreads = 512, kSmallPer = 4;
+
+template <int kMode, bool kContig, int kOut>
+__global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads, 1)
+quantize_small_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, int64_t ldx,
+                      uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, float* tensor_scale, int xr) {
+  __shared__ float4 tab[128];
+  __shared__ uint32_t red[kSmallThreads / 32], maxes[kSmallCtas], amax;
+  griddep_wait();
+  griddep_launch_dependents();
+  const int64_t b0 = (int64_t)blockIdx.x * kSmallThreads + threadIdx.x;
+  constexpr int64_t kStride = (int64_t)kSmallCtas * kSmallThreads;
+  const int64_t ntotal = kOut == 1 ? xr * kblocks : nblocks;
+  uint32_t w[kSmallPer][8], m = 0u;
+#pragma unroll
+  for (int i = 0; i < kSmallPer; ++i) {
+    const int64_t b = b0 + i * kStride;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w[i][j] = 0u;
+    if (b < nblocks) ldg256_stream(block_src<kContig>(x, b, kblocks, ldx), w[i]);
+  }
+  fill_scale_table(tab);
+#pragma unroll
+  for (int i = 0; i < kSmallPer; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) m = __vmaxu2(m, w[i][j] & 0x7FFF7FFFu);
+  m = max(m & 0xFFFFu, m >> 16);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    m = __reduce_max_sync(0xffffffffu, threadIdx.x < kSmallThreads / 32 ? red[threadIdx.x] : 0u);
+    if (threadIdx.x < kSmallCtas)
+      sm100::st_cluster_u32(sm100::mapa_shared(sm100::smem_u32(&maxes[blockIdx.x % kSmallCtas]), threadIdx.x), m);
+  }
+  sm100::cluster_sync();
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kSmallCtas; ++i) m = max(m, maxes[i]);
+    amax = m << 16;
+  }
+  __syncthreads();
+  const TensorConsts tc = tensor_consts(tensor_scale, &amax, 0);
+  const bool markstein = markstein_needed(tc);
+#pragma unroll
+  for (int i = 0; i < kSmallPer; ++i) {
+    const int64_t b = b0 + i * kStride;
+    if (b >= ntotal) break;
+    uint32_t lo, hi, sb;
+    if (tc.scaled) quantize_block<kMode, true, true>(w[i], tc, tab, lo, hi, sb);
+    else if (markstein) quantize_block<kMode, false, true>(w[i], tc, tab, lo, hi, sb);
+    else quantize_block<kMode, false, false>(w[i], tc, tab, lo, hi, sb);
+    if (kOut == 0) {
+      stg64(codes + b * 8, lo, hi);
+      scales[b] = (uint8_t)sb;
+    } else {
+      const int r = (int)(b / kblocks), c = (int)(b - (int64_t)r * kblocks);
+      if (b >= nblocks) lo = hi = sb = 0u;
+      const uint32_t e1m2 = (sb & 0x80u) ? 0xFFFFFFFFu : 0u;
+      stg64(codes + b * 8, lo, hi);
+      stg64(codes + (xr * kblocks + b) * 8, residual_word(lo) & e1m2, residual_word(hi) & e1m2);
+      uint8_t* t = scales + (int64_t)(c / 4) * 512 + (c & 3);
+      t[tiled_scale_row(r)] = (uint8_t)(sb & 0x7Fu);
+      t[tiled_scale_row(xr + r)] = (uint8_t)(sb & 0x7Fu);
+    }
+  }
 }
 
 // Rotation + Algorithm 1, two blocks per thread side by side (as in
@@ -339,6 +416,43 @@ int launch_quantize(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uin
                     int scale_given, cudaStream_t stream) {
   launch_quantize_to<false>(x, rows, K, ldx, codes, scales, tensor_scale, amax_word, mode, scale_given, stream);
   return 0;
+}
+
+namespace {
+
+template <int kOut>
+bool launch_small(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* codes, uint8_t* scales,
+                  float* tensor_scale, int mode, int xr, cudaStream_t stream) {
+  const int64_t kblocks = K / 16, nblocks = rows * kblocks;
+  if ((kOut == 1 ? xr * kblocks : nblocks) > (int64_t)kSmallCtas * kSmallThreads * kSmallPer) return false;
+#define MIXFP4_LAUNCH_SM(MODE)                                                                                  \
+  (ldx == K ? launch_pdl(quantize_small_kernel<MODE, true, kOut>, kSmallCtas, kSmallThreads, 0, stream, x, nblocks, \
+                         kblocks, ldx, codes, scales, tensor_scale, xr)                                          \
+            : launch_pdl(quantize_small_kernel<MODE, false, kOut>, kSmallCtas, kSmallThreads, 0, stream, x, nblocks, \
+                         kblocks, ldx, codes, scales, tensor_scale, xr))
+  switch (mode) {
+    case MIXFP4_MODE_MIX: MIXFP4_LAUNCH_SM(MIXFP4_MODE_MIX); break;
+    case MIXFP4_MODE_E2M1_ONLY: MIXFP4_LAUNCH_SM(MIXFP4_MODE_E2M1_ONLY); break;
+    case MIXFP4_MODE_FOUR_SIX: MIXFP4_LAUNCH_SM(MIXFP4_MODE_FOUR_SIX); break;
+    default: MIXFP4_LAUNCH_SM(MIXFP4_MODE_E1M2_ONLY); break;
+  }
+#undef MIXFP4_LAUNCH_SM
+  return true;  // a launch error is the caller's cudaGetLastError
+}
+
+}  // namespace
+
+// Quantize with the scale computed, in one launch; false (nothing enqueued) for
+// a tensor too large for it.
+bool launch_quantize_small(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* codes, uint8_t* scales,
+                           float* tensor_scale, int mode, cudaStream_t stream) {
+  return launch_small<0>(x, rows, K, ldx, codes, scales, tensor_scale, mode, 0, stream);
+}
+
+// The same into the few-row GEMM's activation operand.
+bool launch_quantize_fewrows(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* xop, uint8_t* sfa,
+                             float* tensor_scale, int mode, int xr, cudaStream_t stream) {
+  return launch_small<1>(x, rows, K, ldx, xop, sfa, tensor_scale, mode, xr, stream);
 }
 
 // The quantized tensor as f16 values u * s8, [rows][K] (the operand of launch_gemm_f16a).

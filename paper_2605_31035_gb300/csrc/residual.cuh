@@ -24,6 +24,10 @@ __device__ __forceinline__ uint32_t residual_word(uint32_t w) {
   return d;
 }
 
+// Byte offset of row r's four ue4m3 scales of a K step in the tensor core's tiled
+// layout of 128 rows.
+__device__ __forceinline__ uint32_t tiled_scale_row(int r) { return (uint32_t)((r & 31) * 16 + (r >> 5) * 4); }
+
 // All ones where block b (0..3) of the four scale bytes s4 is E1M2, else 0
 // (prmt with the sign-replicate selectors).
 __device__ __forceinline__ uint32_t type_mask(uint32_t s4, int b) {

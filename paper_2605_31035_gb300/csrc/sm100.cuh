@@ -83,6 +83,9 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t saddr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(saddr), "r"(rank));
   return d;
 }
+__device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(cluster_addr), "r"(v) : "memory");
+}
 // Arrive on an mbarrier given by a shared::cluster address (local or peer CTA).
 // The release is CTA-scoped: every use signals data that already sits,
 // complete, in the arriving CTA's own shared or tensor memory (a TMA stage
