@@ -215,84 +215,145 @@ quantize_2d_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t K, int6
 // is applied to both WGRAD operands, whose reduction runs over tokens): every
 // 128-row chunk of each column is rotated (reading R11: the caller's sign
 // vector, the same butterfly order) and the rotated column is quantized down
-// its rows -- bit for bit mixfp4_quantize_rht of X^T.  A CTA stages a
-// 128-row x 64-column tile TRANSPOSED in shared memory (a column's 128 values
-// contiguous, 272-byte pitch): each warp loads 8 columns of 32 consecutive
-// rows (16-byte loads) and scatters them with 2-byte stores that are
-// consecutive within the warp.  Then each 8-lane group holds one column chunk
-// (lane b: rows 16b..16b+15, one 32-byte shared read) and rotates it with the
-// row-wise kernel's shuffle butterfly.  kAmax: the pass that reduces max |y|
-// of the rotated tensor into the workspace word instead of quantizing.
-constexpr int kCrRows = 128, kCrCols = 64, kCrPitch = kCrRows + 8;  // staged column pitch (u16)
+// its rows -- bit for bit mixfp4_quantize_rht of X^T.
+//
+// A warp takes 128-row x 16-column tiles on its own (no barriers beyond the
+// warp's).  The butterfly works on pairs of adjacent columns, which are the
+// halves of a loaded word, so the packed fp32 instructions need no shuffles and
+// no transposition: a lane loads 16 rows of a column pair and does strides 1 to
+// 8 in registers; the values pass through the warp's shared memory (fp32, 8
+// bytes a pair); a lane then holds the 8 values 16 rows apart for strides 16 to
+// 64.  kAmax stops there with the maximum; otherwise they pass through shared
+// memory once more and a lane quantizes the two 16-row blocks of a column pair,
+// four lanes side by side on 32 code bytes of a column.  A block of 16 rows
+// starts 272 words after the one before, so that none of the three access
+// patterns (16 lanes of 8 bytes each) conflicts.
+// Against the former form (bf16 tile scattered by 2-byte stores, 48 shuffles a
+// block, CTA barriers) on 4096 x 4096: amax pass 21.3 -> 13.0 us, quantize 31.1
+// -> 25.0 us, both on 8192 x 8192 193 -> 131 us; CTA-wide 64-column tiles of this
+// form: 14.8 and 29.0 us.  Four CTAs per SM: 128 registers, no spills (five or
+// six spill: 41 us for both passes against 38).
+constexpr int kCrRows = 128, kCrCols = 16, kCrWarps = 4, kCrBlk = 16 * kCrCols + 16, kCrTile = 8 * kCrBlk;
+__device__ __forceinline__ int cr_word(int b, int i, int col) { return b * kCrBlk + i * kCrCols + col; }
+
+// One radix-2 stage: strides of h over v[0..n).
+template <int n, int h>
+__device__ __forceinline__ void butterfly(u64 (&v)[n]) {
+#pragma unroll
+  for (int i = 0; i < n; ++i)
+    if ((i & h) == 0) {
+      const u64 a = v[i], b = v[i + h];
+      v[i] = add2(a, b);
+      v[i + h] = sub2(a, b);
+    }
+}
 
 template <int kMode, bool kAmax>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(32 * kCrWarps, 4)
 quantize_colwise_rht_kernel(const uint16_t* __restrict__ x, int64_t R, int64_t C, int64_t ldx,
                             const uint8_t* __restrict__ signs, uint8_t* __restrict__ codes,
                             uint8_t* __restrict__ scales, float* tensor_scale, uint32_t* amax_word, int scale_given) {
   __shared__ float4 tab[128];
-  __shared__ __align__(16) uint16_t tile[kCrCols][kCrPitch];
+  __shared__ __align__(16) float tiles_s[kCrWarps][kCrTile];
   griddep_wait();
   griddep_launch_dependents();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint32_t sw[8];
-  rht_sign_words(signs, lane, sw);  // lane & 7 = the block of the chunk this lane holds
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int cp = lane & 7, g = lane >> 3;  // column pair, and which of four blocks / residues
+  float* tile = tiles_s[warp];
+  uint32_t bits[2] = {0u, 0u};  // sign bits of the 16 rows of blocks g and g + 4 of a chunk
+  if (signs)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      bits[h] = (uint32_t)__ldg(signs + 2 * (g + 4 * h)) | ((uint32_t)__ldg(signs + 2 * (g + 4 * h) + 1) << 8);
   TensorConsts tc{};
   if (!kAmax) {
     fill_scale_table(tab);
     tc = tensor_consts(tensor_scale, amax_word, scale_given);
-  }
-  uint32_t m = 0;
-  const int64_t ct_n = (C + kCrCols - 1) / kCrCols, rt_n = R / kCrRows;
-  for (int64_t t = blockIdx.x; t < ct_n * rt_n; t += gridDim.x) {
-    const int64_t r0 = (t / ct_n) * kCrRows, c0 = (t % ct_n) * kCrCols;
-    // Stage: chunk q = (8 columns from 8 cg, row q % 128).
-#pragma unroll
-    for (int k = 0; k < kCrRows * kCrCols / 8 / 256; ++k) {
-      const int q = tid + 256 * k, row = q & (kCrRows - 1), cg = q >> 7;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (c0 + cg * 8 < C) v = __ldg(reinterpret_cast<const uint4*>(x + (r0 + row) * ldx + c0 + cg * 8));
-      const uint32_t e[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        tile[cg * 8 + 2 * i][row] = (uint16_t)(e[i] & 0xFFFFu);
-        tile[cg * 8 + 2 * i + 1][row] = (uint16_t)(e[i] >> 16);
-      }
-    }
     __syncthreads();
-#pragma unroll 1
-    for (int pass = 0; pass < kCrCols / 32; ++pass) {
-      const int cl = pass * 32 + warp * 4 + (lane >> 3), b = lane & 7;
-      const int64_t c = c0 + cl;
-      const uint4 lo4 = *reinterpret_cast<const uint4*>(&tile[cl][16 * b]);
-      const uint4 hi4 = *reinterpret_cast<const uint4*>(&tile[cl][16 * b + 8]);
-      const uint32_t w[8] = {lo4.x, lo4.y, lo4.z, lo4.w, hi4.x, hi4.y, hi4.z, hi4.w};
-      u64 y[8];
-      rht_rotate(w, sw, lane, y);  // all 32 lanes: shuffles within 8-lane groups
-      if (kAmax) {
+  }
+  const float c128 = __uint_as_float(kRhtScaleBits);
+  const u64 cc = pack2(c128, c128);
+  uint32_t m = 0;
+  const int64_t ct_n = C / kCrCols, tiles = ct_n * (R / kCrRows);
+  const int64_t nwarps = (int64_t)gridDim.x * kCrWarps;
+  for (int64_t t = (int64_t)blockIdx.x * kCrWarps + warp; t < tiles; t += nwarps) {
+    const int64_t rt = t / ct_n, c0 = (t - rt * ct_n) * kCrCols;
+    const uint16_t* src = x + rt * kCrRows * ldx + c0 + 2 * cp;
+    uint32_t w[2][16];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) m = max(m, max(lo32(y[j]) & 0x7FFFFFFFu, hi32(y[j]) & 0x7FFFFFFFu));
-      } else {
-        uint32_t lo, hi, sb;
-        if (tc.scaled) rht_block<kMode, true>(y, tc, tab, lo, hi, sb);
-        else rht_block<kMode, false>(y, tc, tab, lo, hi, sb);
-        if (c < C) {
-          const int64_t ob = r0 / 16 + b;
-          stg64(codes + c * (R / 2) + ob * 8, lo, hi);
-          scales[c * (R / 16) + ob] = (uint8_t)sb;
-        }
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        w[h][i] = __ldg(reinterpret_cast<const uint32_t*>(src + (16 * (g + 4 * h) + i) * ldx));
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {  // strides 1 to 8 of blocks g and g + 4
+      u64 v[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const uint32_t u = w[h][i] ^ (((bits[h] >> i) & 1u) ? 0x80008000u : 0u);
+        v[i] = bits2(u << 16, u & 0xFFFF0000u);
+      }
+      butterfly<16, 1>(v);
+      butterfly<16, 2>(v);
+      butterfly<16, 4>(v);
+      butterfly<16, 8>(v);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) *reinterpret_cast<u64*>(&tile[cr_word(g + 4 * h, i, 2 * cp)]) = v[i];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {  // strides 16 to 64 of rows i, 16 + i, ..., 112 + i
+      const int i = g + 4 * k;
+      u64 v[8];
+#pragma unroll
+      for (int b = 0; b < 8; ++b) v[b] = *reinterpret_cast<const u64*>(&tile[cr_word(b, i, 2 * cp)]);
+      butterfly<8, 1>(v);
+      butterfly<8, 2>(v);
+      butterfly<8, 4>(v);
+#pragma unroll
+      for (int b = 0; b < 8; ++b) {
+        v[b] = mul2(v[b], cc);
+        if (kAmax) m = max(m, max(lo32(v[b]) & 0x7FFFFFFFu, hi32(v[b]) & 0x7FFFFFFFu));
+        else *reinterpret_cast<u64*>(&tile[cr_word(b, i, 2 * cp)]) = v[b];
       }
     }
-    __syncthreads();  // the tile is restaged next
+    __syncwarp();
+    if (!kAmax) {
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        const int b = g + 4 * h;
+        u64 y0[8], y1[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float2 p = *reinterpret_cast<const float2*>(&tile[cr_word(b, 2 * j, 2 * cp)]);
+          const float2 q = *reinterpret_cast<const float2*>(&tile[cr_word(b, 2 * j + 1, 2 * cp)]);
+          y0[j] = pack2(p.x, q.x);
+          y1[j] = pack2(p.y, q.y);
+        }
+        uint32_t lo0, hi0, sb0, lo1, hi1, sb1;
+        if (tc.scaled) {
+          rht_block<kMode, true>(y0, tc, tab, lo0, hi0, sb0);
+          rht_block<kMode, true>(y1, tc, tab, lo1, hi1, sb1);
+        } else {
+          rht_block<kMode, false>(y0, tc, tab, lo0, hi0, sb0);
+          rht_block<kMode, false>(y1, tc, tab, lo1, hi1, sb1);
+        }
+        const int64_t c = c0 + 2 * cp, ob = rt * (kCrRows / 16) + b;
+        stg64(codes + c * (R / 2) + ob * 8, lo0, hi0);
+        stg64(codes + (c + 1) * (R / 2) + ob * 8, lo1, hi1);
+        scales[c * (R / 16) + ob] = (uint8_t)sb0;
+        scales[(c + 1) * (R / 16) + ob] = (uint8_t)sb1;
+      }
+      __syncwarp();  // the tile is rewritten next
+    }
   }
   if (kAmax) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    __shared__ uint32_t red[8];
+    m = __reduce_max_sync(0xffffffffu, m);
+    __shared__ uint32_t red[kCrWarps];
     if (lane == 0) red[warp] = m;
     __syncthreads();
-    if (tid == 0) {
-      for (int i = 1; i < 8; ++i) m = max(m, red[i]);
+    if (threadIdx.x == 0) {
+      for (int i = 1; i < kCrWarps; ++i) m = max(m, red[i]);
       if (m) atomicMax(amax_word, m);
     }
   }
@@ -468,13 +529,14 @@ int launch_quantize_2d(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, 
 int launch_quantize_colwise_rht(const uint16_t* x, int64_t R, int64_t C, int64_t ldx, const uint8_t* signs,
                                 uint8_t* codes, uint8_t* scales, float* tensor_scale, uint32_t* amax_word, int mode,
                                 int scale_given, int amax_pass, cudaStream_t stream) {
-  const int64_t tiles = ((C + kCrCols - 1) / kCrCols) * (R / kCrRows);
-  if (tiles == 0) return 0;
-  const int64_t grid = tiles < num_sms() * 3 ? tiles : num_sms() * 3;
+  const int64_t ctas = (C / kCrCols * (R / kCrRows) + kCrWarps - 1) / kCrWarps;  // C is a multiple of 16
+  if (ctas == 0) return 0;
+  const int64_t cap = num_sms() * 4;
+  const int64_t grid = ctas < cap ? ctas : cap;
   cudaError_t e;
 #define MIXFP4_LAUNCH_CR(MODE, AMAX)                                                                           \
-  e = launch_pdl(quantize_colwise_rht_kernel<MODE, AMAX>, (unsigned)grid, 256, 0, stream, x, R, C, ldx, signs, codes, \
-                 scales, tensor_scale, amax_word, scale_given)
+  e = launch_pdl(quantize_colwise_rht_kernel<MODE, AMAX>, (unsigned)grid, 32 * kCrWarps, 0, stream, x, R, C, ldx, signs, \
+                 codes, scales, tensor_scale, amax_word, scale_given)
   if (amax_pass) {
     MIXFP4_LAUNCH_CR(MIXFP4_MODE_MIX, true);
   } else {
