@@ -91,17 +91,17 @@ __global__ void __launch_bounds__(256) split_native_kernel(const uint8_t* __rest
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_code + n_sf;
        i += (int64_t)gridDim.x * blockDim.x) {
     if (i < n_code) {
-      const int64_t r = i / (K / 32), c = i % (K / 32);  // row, 32-element chunk
-      const uint4 w = *reinterpret_cast<const uint4*>(codes + r * (K / 2) + c * 16);
-      const uint8_t s0 = scales[r * nb + 2 * c], s1 = scales[r * nb + 2 * c + 1];
+      // Rows are dense, so the 32-element chunk i needs no row and column.
+      const uint4 w = *reinterpret_cast<const uint4*>(codes + i * 16);
+      const uint8_t s0 = scales[2 * i], s1 = scales[2 * i + 1];
       const uint32_t k0 = (s0 & 0x80u) ? 0xFFFFFFFFu : 0u, k1 = (s1 & 0x80u) ? 0xFFFFFFFFu : 0u;
       uint4 m, q;
       split_e1m2_word(w.x, k0, m.x, q.x);
       split_e1m2_word(w.y, k0, m.y, q.y);
       split_e1m2_word(w.z, k1, m.z, q.z);
       split_e1m2_word(w.w, k1, m.w, q.w);
-      *reinterpret_cast<uint4*>(main_codes + r * (K / 2) + c * 16) = m;
-      *reinterpret_cast<uint4*>(res_codes + r * (K / 2) + c * 16) = q;
+      *reinterpret_cast<uint4*>(main_codes + i * 16) = m;
+      *reinterpret_cast<uint4*>(res_codes + i * 16) = q;
     } else {
       const int64_t u = i - n_code;
       const int64_t line = u % 32, tile = u / 32, kt_n = K / 64;
