@@ -299,8 +299,8 @@ int mixfp4_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_
  *              K % 256 == 0 as mixfp4_gemm's.
  * w_codes/w_scales/w_ts      W, N x K, as mixfp4_gemm's B.
  * C, ldc, status_word        as mixfp4_gemm's.
- * workspace    device, 256-byte aligned, at least 2 M K + 512 bytes; written by the
- *              call and free for reuse once the call's work on `stream` is done.
+ * workspace    device, 256-byte aligned, at least 2 M K + 16384 bytes; written by
+ *              the call and free for reuse once the call's work on `stream` is done.
  *              With the bytes mixfp4_linear_workspace reports, a long K may be cut
  *              into parts that run side by side (their sum is compensated).
  * workspace_bytes  its size.
@@ -312,7 +312,7 @@ int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, i
 
 /*
  * mixfp4_linear_workspace -- bytes of workspace mixfp4_linear makes use of, at
- * least the 2 M K + 512 it needs, on the current device.
+ * least the 2 M K + 16384 it needs, on the current device.
  *
  * bytes        host, one int64.                                          (output)
  */

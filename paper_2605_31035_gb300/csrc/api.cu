@@ -303,9 +303,15 @@ int64_t gemm_scratch(int64_t M, int64_t N, int64_t K) {
   return M * K * 2 + mixfp4::gemm_f16a_parts_bytes(M, N, K);
 }
 
-// mixfp4_linear's scratch for up to 64 rows: amax word and s32 (256 bytes), the
-// codes, the block scales, then (at the returned offset) launch_fewrows' own.
-int64_t few_rows_offset(int64_t M, int64_t K) { return (256 + M * (K / 2) + M * (K / 16) + 255) / 256 * 256; }
+// mixfp4_linear's scratch: the maxima of the amax pass, then s32 (256 bytes),
+// then the quantized activations.
+constexpr int64_t kLinearHeader = mixfp4::kMaxAmaxParts * 4 + 256;
+constexpr int64_t kLinearExtra = 16384;  // bytes mixfp4_linear needs beyond 2 M K (mixfp4.h)
+static_assert(kLinearHeader <= kLinearExtra, "linear workspace");
+
+// Up to 64 rows: the codes, the block scales, then (at the returned offset)
+// launch_fewrows' own scratch.
+int64_t few_rows_offset(int64_t M, int64_t K) { return (kLinearHeader + M * (K / 2) + M * (K / 16) + 255) / 256 * 256; }
 
 // Shared body of the decode-path GEMM entry points.
 int gemm_impl(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts, const uint8_t* b_codes,
@@ -375,7 +381,7 @@ int mixfp4_linear_workspace(int64_t M, int64_t N, int64_t K, int64_t* bytes) {
   if (!bytes) return MIXFP4_ERR_NULL;
   if (M < 0 || N < 0 || K < 0 || K % 256 != 0) return MIXFP4_ERR_SHAPE;
   if (M > (1 << 30) || N > (1 << 30) || K > (1 << 30)) return MIXFP4_ERR_SHAPE;
-  *bytes = 2 * M * K + 512;
+  *bytes = 2 * M * K + kLinearExtra;
   if (M == 0 || N == 0 || K == 0) return MIXFP4_OK;
   if (M > 64) {
     *bytes += mixfp4::gemm_f16a_parts_bytes(M, N, K);
@@ -397,12 +403,12 @@ int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, i
   }
   if (!workspace) return MIXFP4_ERR_NULL;
   if (!aligned(workspace, 256)) return MIXFP4_ERR_ALIGN;
-  if (M > (1 << 30) || N > (1 << 30) || K > (1 << 30) || workspace_bytes < 2 * M * K + 512) return MIXFP4_ERR_SHAPE;
-  // Scratch: the amax word and s32, then the quantized activations: decoded to
-  // f16 for the GEMM that takes A so, as codes and block scales for few rows.
-  uint32_t* amax_word = static_cast<uint32_t*>(workspace);
-  float* x_ts = static_cast<float*>(workspace) + 4;
-  uint8_t* xq = static_cast<uint8_t*>(workspace) + 256;
+  if (M > (1 << 30) || N > (1 << 30) || K > (1 << 30) || workspace_bytes < 2 * M * K + kLinearExtra) return MIXFP4_ERR_SHAPE;
+  // Quantized activations: decoded to f16 for the GEMM that takes A so, as codes
+  // and block scales (or the few-row GEMM's operand) for few rows.
+  uint32_t* amax_words = static_cast<uint32_t*>(workspace);
+  float* x_ts = static_cast<float*>(workspace) + mixfp4::kMaxAmaxParts;
+  uint8_t* xq = static_cast<uint8_t*>(workspace) + kLinearHeader;
   if (dtype != MIXFP4_DTYPE_BF16) return MIXFP4_ERR_DTYPE;
   if (mode < MIXFP4_MODE_MIX || mode > MIXFP4_MODE_FOUR_SIX) return MIXFP4_ERR_ARG;
   if (!x || !w_codes || !w_scales || !w_ts || !C) return MIXFP4_ERR_NULL;
@@ -421,18 +427,15 @@ int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, i
                                       status_word, s, &st))
       return st ? st : launch_status();
     uint8_t* x_scales = xq + M * (K / 2);  // K / 2 is a multiple of 128
-    st = mixfp4_quantize(x, dtype, M, K, ldx, xq, x_scales, x_ts, amax_word, mode, MIXFP4_SCALE_COMPUTE, stream);
+    st = mixfp4_quantize(x, dtype, M, K, ldx, xq, x_scales, x_ts, amax_words, mode, MIXFP4_SCALE_COMPUTE, stream);
     if (st) return st;
     return mixfp4_gemm_ws(xq, x_scales, x_ts, w_codes, w_scales, w_ts, M, N, K, C, ldc, scratch, room, status_word,
                           stream);
   }
-  if (cudaMemsetAsync(amax_word, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
-  mixfp4::launch_amax(xb, M, K, ldx, amax_word, s);
-  if (int st = launch_status()) return st;
-  mixfp4::launch_quantize_f16(xb, M, K, ldx, xq, x_ts, amax_word, mode, s);
+  mixfp4::launch_quantize_f16(xb, M, K, ldx, xq, x_ts, amax_words, mode, s);
   if (int st = launch_status()) return st;
   if (int st = mixfp4::launch_gemm_f16a(xq, x_ts, w_codes, w_scales, w_ts, M, N, K, C, ldc, xq + M * K * 2,
-                                        workspace_bytes - M * K * 2 - 256, status_word, s))
+                                        workspace_bytes - M * K * 2 - kLinearHeader, status_word, s))
     return st;
   return launch_status();
 }

@@ -17,8 +17,9 @@ bool launch_quantize_small(const uint16_t* x, int64_t rows, int64_t K, int64_t l
                            float* tensor_scale, int mode, cudaStream_t stream);
 bool launch_quantize_fewrows(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* xop, uint8_t* sfa,
                              float* tensor_scale, int mode, int xr, cudaStream_t stream);
+constexpr int kMaxAmaxParts = 2048;  // maxima of launch_quantize_f16's first pass
 int launch_quantize_f16(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, void* out, float* tensor_scale,
-                        const uint32_t* amax_word, int mode, cudaStream_t stream);
+                        uint32_t* parts, int mode, cudaStream_t stream);
 int launch_rht_amax(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, const uint8_t* signs,
                     uint32_t* amax_word, cudaStream_t stream);
 int launch_rht_quantize(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, const uint8_t* signs,

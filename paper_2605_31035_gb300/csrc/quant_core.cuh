@@ -285,25 +285,28 @@ __device__ __forceinline__ void block_core(const u64 a[8], const TensorConsts& t
     const u64 nmagic = pack2(-12582912.0f, -12582912.0f);
     const bool clamp = !(t.x >= 0x1p-6f && b7 <= 448.0f);
     u64 acc = 0;
-    uint32_t pb[8];
+    const u64 k256 = pack2(256.0f, 256.0f);
+    uint32_t even[4], odd[4];  // payloads of two pairs' even (odd) elements at bits 0 and 8
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const u64 y = div_kd2(a[j], zh8, zl8);
-      const u64 tq = add2(y, magic);  // RNE to an integer in the low mantissa bits
-      uint32_t tlo = lo32(tq), thi = hi32(tq);
-      if (clamp) {
-        tlo = min(tlo, 0x4B400007u);
-        thi = min(thi, 0x4B400007u);
+    for (int g = 0; g < 4; ++g) {
+      u64 q[2], tq[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int j = 2 * g + i;
+        tq[i] = add2(div_kd2(a[j], zh8, zl8), magic);  // RNE to an integer in the low mantissa bits
+        if (clamp) tq[i] = bits2(min(lo32(tq[i]), 0x4B400007u), min(hi32(tq[i]), 0x4B400007u));
+        q[i] = add2(tq[i], nmagic);
+        if (kMode == MIXFP4_MODE_MIX) {
+          const u64 d = fma2(q[i], ns8, a[j]);
+          acc = fma2(d, d, acc);
+        }
       }
-      pb[j] = tlo + (thi << 4);  // low byte: payload pair (first element low)
-      if (kMode == MIXFP4_MODE_MIX) {
-        const u64 q = add2(bits2(tlo, thi), nmagic);
-        const u64 d = fma2(q, ns8, a[j]);
-        acc = fma2(d, d, acc);
-      }
+      const u64 both = fma2(q[1], k256, tq[0]);  // exact: magic + q0 + 256 q1
+      even[g] = lo32(both);
+      odd[g] = hi32(both);
     }
-    p1lo = pack_low_bytes(pb[0], pb[1], pb[2], pb[3]);
-    p1hi = pack_low_bytes(pb[4], pb[5], pb[6], pb[7]);
+    p1lo = prmt(even[0], even[1], 0x5410u) + (prmt(odd[0], odd[1], 0x5410u) << 4);
+    p1hi = prmt(even[2], even[3], 0x5410u) + (prmt(odd[2], odd[3], 0x5410u) << 4);
     if (kMode == MIXFP4_MODE_MIX) {
       float se, so;
       unpack2(acc, se, so);

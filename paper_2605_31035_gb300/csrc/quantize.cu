@@ -68,15 +68,18 @@ __device__ __forceinline__ void store_block(uint8_t* __restrict__ codes, uint8_t
 // at a time (a, b): both blocks of a pair are quantized before either is
 // stored, so their independent dependency chains interleave, and the loads of
 // the next pair are in flight meanwhile.  The division method is fixed per
-// launch, so each method gets its own copy of the loop.
-template <int kMode, bool kContig, bool kF16, bool kScaled, bool kMarkstein>
-__device__ __forceinline__ void quantize_pairs(const uint16_t* __restrict__ x, int64_t b, int64_t nthr,
-                                               int64_t nblocks, int64_t kblocks, int64_t ldx,
+// launch, so each method gets its own copy of the loop; the usual one runs on
+// 32-bit block indices where they suffice (2^28 elements 177 -> 170 us: the
+// kernel is bound by instruction issue, and 64-bit index arithmetic was one
+// instruction in thirty).
+template <int kMode, bool kContig, bool kF16, bool kScaled, bool kMarkstein, typename Index>
+__device__ __forceinline__ void quantize_pairs(const uint16_t* __restrict__ x, Index b, Index nthr,
+                                               Index nblocks, int64_t kblocks, int64_t ldx,
                                                uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
                                                const TensorConsts& tc, const float4* __restrict__ tab,
                                                uint32_t (&wa)[8], uint32_t (&wb)[8]) {
   for (; b < nblocks; b += 2 * nthr) {
-    const int64_t b1 = b + nthr;
+    const Index b1 = b + nthr;
     uint32_t lo0, hi0, sb0, lo1, hi1, sb1;
     quantize_block<kMode, kScaled, kMarkstein>(wa, tc, tab, lo0, hi0, sb0);
     quantize_block<kMode, kScaled, kMarkstein>(wb, tc, tab, lo1, hi1, sb1);  // wb past the end: unused
@@ -94,7 +97,7 @@ template <int kMode, bool kContig, bool kF16>
 __global__ void __launch_bounds__(kQuantThreads, 4)
 quantize_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, int64_t ldx,
                 uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, float* tensor_scale,
-                const uint32_t* amax_word, int scale_given, int after_amax) {
+                const uint32_t* amax_word, int amax_parts, int scale_given, int after_amax) {
   __shared__ float4 tab[128];  // E4M3 code -> {s8, zh, zl, 0} (zh, zl: see div_kd2)
   // Launched as a programmatic dependent of the amax kernel (after_amax), x
   // is already complete and may be read before that kernel finishes; only
@@ -110,14 +113,31 @@ quantize_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks
   if (b + nthr < nblocks) ldg256_stream(block_src<kContig>(x, b + nthr, kblocks, ldx), wb);
   fill_scale_table(tab);
   if (after_amax) griddep_wait();
+  if (kF16) {
+    // The amax pass's maxima, one per CTA of it.
+    __shared__ uint32_t red[kQuantThreads / 32];
+    uint32_t m = 0u;
+    for (int i = threadIdx.x; i < amax_parts; i += kQuantThreads) m = max(m, __ldcg(amax_word + i));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kQuantThreads / 32; ++i) m = max(m, red[i]);
+    __syncthreads();
+    if (threadIdx.x == 0) red[0] = m;
+    __syncthreads();
+    amax_word = red;
+  }
   const TensorConsts tc = tensor_consts(tensor_scale, amax_word, scale_given);
   const bool markstein = markstein_needed(tc);
   if (tc.scaled)
-    quantize_pairs<kMode, kContig, kF16, true, true>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
+    quantize_pairs<kMode, kContig, kF16, true, true, int64_t>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
   else if (markstein)
-    quantize_pairs<kMode, kContig, kF16, false, true>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
+    quantize_pairs<kMode, kContig, kF16, false, true, int64_t>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
+  else if (nblocks < (1ll << 30))
+    quantize_pairs<kMode, kContig, kF16, false, false, uint32_t>(x, (uint32_t)b, (uint32_t)nthr, (uint32_t)nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
   else
-    quantize_pairs<kMode, kContig, kF16, false, false>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
+    quantize_pairs<kMode, kContig, kF16, false, false, int64_t>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, wa, wb);
 }
 
 // Small tensors in one launch: a cluster of eight CTAs holds the whole tensor in
@@ -195,6 +215,36 @@ quantize_small_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t k
   }
 }
 
+template <int kMode, bool kContig, typename Index>
+__device__ __forceinline__ void rht_pairs(const uint16_t* __restrict__ x, Index b, Index nthr, Index nblocks,
+                                          int64_t kblocks, int64_t ldx, uint8_t* __restrict__ codes,
+                                          uint8_t* __restrict__ scales, const TensorConsts& tc,
+                                          const float4* __restrict__ tab, const uint32_t (&sw)[8], int lane,
+                                          uint32_t (&w)[8], uint32_t (&w2)[8]) {
+  for (; b < nblocks; b += 2 * nthr) {
+    const Index b1 = b + nthr;
+    u64 y[8], y2[8];
+    rht_rotate(w, sw, lane, y);
+    rht_rotate(w2, sw, lane, y2);  // the 8 lanes of a chunk agree on b1 < nblocks
+    if (b + 2 * nthr < nblocks) ldg256_stream(block_src<kContig>(x, b + 2 * nthr, kblocks, ldx), w);
+    if (b1 + 2 * nthr < nblocks) ldg256_stream(block_src<kContig>(x, b1 + 2 * nthr, kblocks, ldx), w2);
+    uint32_t lo, hi, sb, lo2, hi2, sb2;
+    if (tc.scaled) {
+      rht_block<kMode, true>(y, tc, tab, lo, hi, sb);
+      rht_block<kMode, true>(y2, tc, tab, lo2, hi2, sb2);
+    } else {
+      rht_block<kMode, false>(y, tc, tab, lo, hi, sb);
+      rht_block<kMode, false>(y2, tc, tab, lo2, hi2, sb2);
+    }
+    stg64(codes + (int64_t)b * 8, lo, hi);
+    scales[b] = (uint8_t)sb;
+    if (b1 < nblocks) {
+      stg64(codes + (int64_t)b1 * 8, lo2, hi2);
+      scales[b1] = (uint8_t)sb2;
+    }
+  }
+}
+
 // Rotation + Algorithm 1, two blocks per thread side by side (as in
 // quantize_kernel); the rotated pairs take 2 CTAs per SM of registers.
 template <int kMode, bool kContig>
@@ -224,28 +274,11 @@ rht_quantize_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kbl
   if (after_amax) griddep_wait();
   const TensorConsts tc = tensor_consts(tensor_scale, amax_word, scale_given);
   __syncthreads();
-  for (; b < nblocks; b += 2 * nthr) {
-    const int64_t b1 = b + nthr;
-    u64 y[8], y2[8];
-    rht_rotate(w, sw, lane, y);
-    rht_rotate(w2, sw, lane, y2);  // the 8 lanes of a chunk agree on b1 < nblocks
-    if (b + 2 * nthr < nblocks) ldg256_stream(block_src<kContig>(x, b + 2 * nthr, kblocks, ldx), w);
-    if (b1 + 2 * nthr < nblocks) ldg256_stream(block_src<kContig>(x, b1 + 2 * nthr, kblocks, ldx), w2);
-    uint32_t lo, hi, sb, lo2, hi2, sb2;
-    if (tc.scaled) {
-      rht_block<kMode, true>(y, tc, tab, lo, hi, sb);
-      rht_block<kMode, true>(y2, tc, tab, lo2, hi2, sb2);
-    } else {
-      rht_block<kMode, false>(y, tc, tab, lo, hi, sb);
-      rht_block<kMode, false>(y2, tc, tab, lo2, hi2, sb2);
-    }
-    stg64(codes + b * 8, lo, hi);
-    scales[b] = (uint8_t)sb;
-    if (b1 < nblocks) {
-      stg64(codes + b1 * 8, lo2, hi2);
-      scales[b1] = (uint8_t)sb2;
-    }
-  }
+  if (nblocks < (1ll << 30))
+    rht_pairs<kMode, kContig, uint32_t>(x, (uint32_t)b, (uint32_t)nthr, (uint32_t)nblocks, kblocks, ldx, codes, scales, tc,
+                                        tab, sw, lane, w, w2);
+  else
+    rht_pairs<kMode, kContig, int64_t>(x, b, nthr, nblocks, kblocks, ldx, codes, scales, tc, tab, sw, lane, w, w2);
 }
 
 // max |y| of the rotated tensor as the bit pattern of a non-negative fp32.
@@ -295,10 +328,14 @@ __device__ __forceinline__ const uint16_t* amax_src(const uint16_t* x, int64_t b
   return x + row * ldx + (b - row * kblocks) * 16;
 }
 
-template <bool kContig>
+// kParts: each CTA leaves its maximum in amax_word[blockIdx.x] for the quantize
+// kernel to reduce, so nothing has to be zeroed first (a memset and its gaps
+// are about 2.5 us of a call).
+template <bool kContig, bool kParts>
 __global__ void __launch_bounds__(256)
 amax_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, int64_t ldx,
             uint32_t* amax_word) {
+  if (kParts) griddep_wait();
   uint32_t m = 0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nblocks; b += kAmaxUnroll * stride) {
@@ -324,7 +361,8 @@ amax_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, in
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = max(m, red[i]);
-    if (m) atomicMax(amax_word, m << 16);
+    if (kParts) amax_word[blockIdx.x] = m << 16;
+    else if (m) atomicMax(amax_word, m << 16);
   }
   // The quantize kernel that follows may start once every CTA got here.
   griddep_launch_dependents();
@@ -371,16 +409,28 @@ int launch_amax(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint32_
   if (nblocks == 0) return 0;
   int64_t grid = (nblocks + 256 * kAmaxUnroll - 1) / (256 * kAmaxUnroll);
   if (grid > num_sms() * 8) grid = num_sms() * 8;
-  if (ldx == K) amax_kernel<true><<<(unsigned)grid, 256, 0, stream>>>(x, nblocks, kblocks, ldx, amax_word);
-  else amax_kernel<false><<<(unsigned)grid, 256, 0, stream>>>(x, nblocks, kblocks, ldx, amax_word);
+  if (ldx == K) amax_kernel<true, false><<<(unsigned)grid, 256, 0, stream>>>(x, nblocks, kblocks, ldx, amax_word);
+  else amax_kernel<false, false><<<(unsigned)grid, 256, 0, stream>>>(x, nblocks, kblocks, ldx, amax_word);
   return 0;
+}
+
+// Maxima of `*n` parts of the tensor into parts[0 .. *n) (*n <= kMaxAmaxParts).
+static void launch_amax_parts(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint32_t* parts, int* n,
+                              cudaStream_t stream) {
+  const int64_t kblocks = K / 16, nblocks = rows * kblocks;
+  int64_t grid = (nblocks + 256 * kAmaxUnroll - 1) / (256 * kAmaxUnroll);
+  if (grid > num_sms() * 8) grid = num_sms() * 8;
+  if (grid > kMaxAmaxParts) grid = kMaxAmaxParts;
+  *n = (int)grid;
+  if (ldx == K) launch_pdl(amax_kernel<true, true>, (unsigned)grid, 256, 0, stream, x, nblocks, kblocks, ldx, parts);
+  else launch_pdl(amax_kernel<false, true>, (unsigned)grid, 256, 0, stream, x, nblocks, kblocks, ldx, parts);
 }
 
 namespace {
 
 template <bool kF16>
 void launch_quantize_to(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* codes, uint8_t* scales,
-                        float* tensor_scale, const uint32_t* amax_word, int mode, int scale_given,
+                        float* tensor_scale, const uint32_t* amax_word, int amax_parts, int mode, int scale_given,
                         cudaStream_t stream) {
   const int64_t kblocks = K / 16, nblocks = rows * kblocks;
   // Persistent grid: 4 CTAs per SM of the device, fewer for small tensors
@@ -395,10 +445,10 @@ void launch_quantize_to(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx,
   do {                                                                                                    \
     if (ldx == K)                                                                                         \
       launch_pdl(quantize_kernel<MODE, true, kF16>, (unsigned)grid, kQuantThreads, 0, stream, x, nblocks,  \
-                 kblocks, ldx, codes, scales, tensor_scale, amax_word, scale_given, after_amax);          \
+                 kblocks, ldx, codes, scales, tensor_scale, amax_word, amax_parts, scale_given, after_amax); \
     else                                                                                                  \
       launch_pdl(quantize_kernel<MODE, false, kF16>, (unsigned)grid, kQuantThreads, 0, stream, x, nblocks, \
-                 kblocks, ldx, codes, scales, tensor_scale, amax_word, scale_given, after_amax);          \
+                 kblocks, ldx, codes, scales, tensor_scale, amax_word, amax_parts, scale_given, after_amax); \
   } while (0)
   switch (mode) {
     case MIXFP4_MODE_MIX: MIXFP4_LAUNCH_Q(MIXFP4_MODE_MIX); break;
@@ -414,7 +464,7 @@ void launch_quantize_to(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx,
 int launch_quantize(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* codes,
                     uint8_t* scales, float* tensor_scale, const uint32_t* amax_word, int mode,
                     int scale_given, cudaStream_t stream) {
-  launch_quantize_to<false>(x, rows, K, ldx, codes, scales, tensor_scale, amax_word, mode, scale_given, stream);
+  launch_quantize_to<false>(x, rows, K, ldx, codes, scales, tensor_scale, amax_word, 0, mode, scale_given, stream);
   return 0;
 }
 
@@ -455,10 +505,13 @@ bool launch_quantize_fewrows(const uint16_t* x, int64_t rows, int64_t K, int64_t
   return launch_small<1>(x, rows, K, ldx, xop, sfa, tensor_scale, mode, xr, stream);
 }
 
-// The quantized tensor as f16 values u * s8, [rows][K] (the operand of launch_gemm_f16a).
+// The tensor quantized with its scale computed, as f16 values u * s8, [rows][K]
+// (the operand of launch_gemm_f16a).  parts: scratch of kMaxAmaxParts words.
 int launch_quantize_f16(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, void* out, float* tensor_scale,
-                        const uint32_t* amax_word, int mode, cudaStream_t stream) {
-  launch_quantize_to<true>(x, rows, K, ldx, static_cast<uint8_t*>(out), nullptr, tensor_scale, amax_word, mode, 0,
+                        uint32_t* parts, int mode, cudaStream_t stream) {
+  int n = 0;
+  launch_amax_parts(x, rows, K, ldx, parts, &n, stream);
+  launch_quantize_to<true>(x, rows, K, ldx, static_cast<uint8_t*>(out), nullptr, tensor_scale, parts, n, mode, 0,
                            stream);
   return 0;
 }
