@@ -22,7 +22,8 @@
 // weight rows, so C is stored coalesced.  Per 64-K step three kind::mxf4nvf4
 // MMAs: the stored codes into D2, the two masked tiles into D1.  Per CTA:
 //   warp 0       TMA: activation operand, weight codes (128-byte swizzle) and
-//                activation scales into the raw ring;
+//                activation scales into the raw ring; the first weight codes
+//                before the activations are ready;
 //   warp 1       TMEM allocator; one thread copies each unit's scales to tensor
 //                memory (tcgen05.cp, about 9 cycles each) and issues its MMAs;
 //   warp 2       the weight rows' block scales, 16 bytes a row, into the raw ring
@@ -156,6 +157,15 @@ fewrows_prep_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict
   }
 }
 
+// Units whose weight codes are requested while the kernel before still writes
+// the activations.  linear() with weights out of L2 (M x N x K, us): 1x14336x4096
+// 20.5 with none, 18.4 with 2, 18.4 with the whole ring; 1x4096x14336 25.4,
+// 23.6, 23.0; 16x28672x8192 44.5, 43.0, 42.5; 20x14336x14336 48.7, 48.1, 49.2.
+// After the shorter operand kernel of a GEMM on quantized rows the whole ring
+// costs up to 0.8 us (1x4096x14336 13.4, 13.5, 14.2: its small loads queue
+// behind the weights), two units nothing.
+constexpr int kAhead = 2;
+
 __global__ void __launch_bounds__(kThreads, 1)
 fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                const uint8_t* __restrict__ w_scales, const uint8_t* __restrict__ sfa, int M, int xr, int N, int K,
@@ -211,27 +221,43 @@ fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
+    // The weights do not depend on the kernel before this one (see the launch),
+    // so the first kAhead units' codes are requested before waiting for it (and
+    // the scale warp does not wait at all); their activation parts follow after
+    // the wait, the other units in one go.
     if (elect_one()) {
       tma_prefetch(&tm_w);
       tma_prefetch(&tm_x);
-      griddep_wait();
       const uint32_t tx = (uint32_t)off_ws(xr);  // all of the stage but the weight scale rows
+      auto load_w = [&](int s, int row, int kc) {
+        const uint32_t fb = smem_u32(&bars->raw_full[s]);
+        mbar_arrive_expect_tx(fb, tx);
+        tma_load_2d(raw0 + (uint32_t)s * RS + (uint32_t)off_w(xr), &tm_w, kc * ROWB, row, fb);
+      };
+      auto load_x = [&](int s, int kc) {
+        const uint32_t st = raw0 + (uint32_t)s * RS, fb = smem_u32(&bars->raw_full[s]);
+        tma_load_2d(st, &tm_x, kc * ROWB, 0, fb);
+        bulk_load(st + (uint32_t)off_sfa(xr), sfa + (int64_t)kc * SF_UNIT, SF_UNIT, fb);
+      };
+      int n = 0;
+      for (int item = blockIdx.x; item < items && n < kAhead; item += gridDim.x)
+        for (int kc = k_begin(item); kc < k_end(item) && n < kAhead; ++kc, ++n) load_w(n, (item / splits) * WR, kc);
+      griddep_wait();
       int it = 0, last = -1, s = 0;
       uint32_t ph = 1;
       bool ok = true;
       for (int item = blockIdx.x; item < items && ok; item += gridDim.x) {
         const int row = (item / splits) * WR, ke = k_end(item);
         for (int kc = k_begin(item); kc < ke; ++kc, ++it) {
-          if (!mbar_wait(smem_u32(&bars->raw_empty[s]), ph, abort_flag, kWaitLimitNs)) {
-            fail(1u);
-            ok = false;
-            break;
+          if (it >= n) {
+            if (!mbar_wait(smem_u32(&bars->raw_empty[s]), ph, abort_flag, kWaitLimitNs)) {
+              fail(1u);
+              ok = false;
+              break;
+            }
+            load_w(s, row, kc);
           }
-          const uint32_t st = raw0 + (uint32_t)s * RS, fb = smem_u32(&bars->raw_full[s]);
-          mbar_arrive_expect_tx(fb, tx);
-          tma_load_2d(st + (uint32_t)off_w(xr), &tm_w, kc * ROWB, row, fb);
-          tma_load_2d(st, &tm_x, kc * ROWB, 0, fb);
-          bulk_load(st + (uint32_t)off_sfa(xr), sfa + (int64_t)kc * SF_UNIT, SF_UNIT, fb);
+          load_x(s, kc);
           last = it;
           if (++s == R) {
             s = 0;
@@ -304,7 +330,6 @@ fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
     }
   } else if (warp == 2) {
     // ---------------- weight scale rows ----------------
-    griddep_wait();
     int s = 0;
     uint32_t ph = 1;
     bool ok = true;
@@ -506,6 +531,10 @@ static int launch_fewrows_main(const float* a_ts, const uint8_t* b_codes, const 
   const int64_t items = tiles * splits;
   const int64_t grid = items < num_sms() ? items : num_sms();
   float* parts = reinterpret_cast<float*>(base + sc.parts);
+  // A programmatic dependent of the kernel that writes the activation operand
+  // (the small quantizer or fewrows_prep_kernel).  That kernel lets this one
+  // start only after its own wait for everything before it, so the weights are
+  // complete here from the start; only what it writes must be waited for.
   if (launch_pdl(fr::fewrows_kernel, (unsigned)grid, fr::kThreads, (size_t)fr::smem_of(xr), stream, tw, tx, b_scales,
                  static_cast<const uint8_t*>(base + sc.sfa), (int)M, xr, (int)N, (int)K, splits, kps, a_ts,
                  b_ts, parts, C, (long long)ldc, status_word) != cudaSuccess)
