@@ -30,7 +30,9 @@
 //                by cp.async (a 16-byte-wide TMA box runs at 0.9 TB/s, and plain
 //                loads in the splitters stall their proxy fence for a DRAM
 //                round trip: 1.5 us a unit);
-//   warps 4-7    epilogue, one TMEM lane quarter each;
+//   warps 4-7    epilogue, one TMEM lane quarter each (for XR = 64, where eight
+//                splitter warps have no slot, twelve warps: three share a
+//                quarter's activation rows in turns of eight);
 //   warps 8-31   three groups of eight (two for XR = 64) taking units in turn,
 //                two threads per weight row: masked codes into tensor memory (the MMA's A
 //                operand; in shared memory their stores and the MMA's reads
@@ -38,7 +40,12 @@
 //                scale tiles (E2M1 blocks, E1M2 blocks) into shared memory.
 // An item adds up D2 + 2 D1 over main and residual columns with two-sum
 // compensation and stores C, or, with K in several parts, its part;
-// sum_parts_kernel adds those up the same way.
+// sum_parts_kernel adds those up the same way.  The sums run on packed fp32
+// pairs, two activation rows an instruction; with the twelve warps that took the
+// GEMM at 64 x 28672 x 8192 from 50.0 to 44.6 us, at 64 x 14336 x 4096 from 16.9
+// to 14.9, at 16 x 28672 x 8192 from 33.3 to 32.1.  (An exchange of the parts
+// within a cluster in place of the sum kernel took 40 us there: its cluster-wide
+// release waits for the loads in flight, 3 us an item.)
 //
 // Every pipeline wait is bounded; a wait that gives up records a status bit
 // (1 producer, 2 / 4 MMA thread, 8 final drain, 16 / 32 splitters, 64
@@ -94,6 +101,8 @@ __host__ __device__ constexpr int split_slots(int xr) { return xr == 64 ? 2 : 3;
 // groups as split slots, and a raw slot's previous landing must lie before the
 // last unit known to be consumed (groups + slots units back).
 __host__ __device__ constexpr int groups(int xr) { return split_slots(xr); }
+// Sets of four epilogue warps: the warps of a group without a slot join warps 4-7.
+__host__ __device__ constexpr int epi_sets(int xr) { return 1 + 2 * (kGroups - groups(xr)); }
 __host__ __device__ constexpr int smem_of(int xr) {
   return 1024 + OFF_RINGS + raw_stages(xr) * raw_stage(xr) + split_slots(xr) * SPLIT_SLOT;
 }
@@ -117,6 +126,13 @@ inline Scratch scratch_of(int64_t M, int64_t N, int64_t K, int splits) {
   s.parts = s.sfa + K / BKC * SF_UNIT;
   s.bytes = s.parts + (splits > 1 ? splits * M * tiles * WR * 4 : 0);
   return s;
+}
+
+// two_sum_add on pairs.
+__device__ __forceinline__ void two_sum_add2(u64& s, u64& e, u64 v) {
+  const u64 t = add2(s, v), z = sub2(t, s);
+  e = add2(e, add2(sub2(s, sub2(t, z)), sub2(v, z)));
+  s = t;
 }
 
 struct Bars {
@@ -192,7 +208,7 @@ fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
     }
     for (int s = 0; s < NB; ++s) {
       mbar_init(smem_u32(&bars->acc_full[s]), 1);
-      mbar_init(smem_u32(&bars->acc_empty[s]), 4);
+      mbar_init(smem_u32(&bars->acc_empty[s]), 4 * (uint32_t)epi_sets(xr));
     }
     mbar_init(smem_u32(&bars->drain), 1);
     bars->abort = 0;
@@ -356,7 +372,7 @@ fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
       ok = __all_sync(0xffffffffu, ok);
     }
     cp_async_wait_all();
-  } else if (warp >= kFirstSplit) {
+  } else if (warp >= kFirstSplit && warp < kFirstSplit + groups(xr) * kGroupWarps) {
     // ---------------- masked code tiles and scale tiles ----------------
     const int g = (warp - kFirstSplit) / kGroupWarps;
     const int row = (warp & 3) * 32 + lane;       // the warp's TMEM lane quarter
@@ -364,7 +380,7 @@ fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
     const uint32_t swz = (uint32_t)(row & 7);
     // Walk of this group's units: every G-th one of the CTA's sequence.
     const int G = groups(xr);
-    int item = g < G ? blockIdx.x : items, kc = k_begin(item), ke = k_end(item), it = 0;
+    int item = blockIdx.x, kc = k_begin(item), ke = k_end(item), it = 0;
     auto advance = [&](int steps) {
       for (; steps > 0 && item < items; --steps, ++it)
         if (++kc >= ke) {
@@ -430,7 +446,9 @@ fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
     const int q = warp & 3;
     griddep_wait();
     const float sa = __ldg(a_ts), sb = __ldg(b_ts);
+    const u64 sa2 = pack2(sa, sa), sb2 = pack2(sb, sb), two = pack2(2.0f, 2.0f);
     const int npad = tiles * WR;
+    const int set = warp < kFirstSplit ? 0 : (warp - kFirstSplit) / 4 - 2 * groups(xr) + 1;
     int ab = 0;
     uint32_t aph = 0;
     for (int item = blockIdx.x; item < items; item += gridDim.x) {
@@ -444,7 +462,7 @@ fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
       const int part = item % splits, n = (item / splits) * WR + q * 32 + lane;
       const uint32_t t2 = tmem_base + (uint32_t)(ab * 4 * xr) + ((uint32_t)(q * 32) << 16), t1 = t2 + (uint32_t)(2 * xr);
 #pragma unroll 1
-      for (int m0 = 0; m0 < M; m0 += 8) {
+      for (int m0 = 8 * set; m0 < M; m0 += 8 * epi_sets(xr)) {
         uint32_t v[4][8];
         tmem_ld_32x32b_x8(t2 + (uint32_t)m0, v[0]);
         tmem_ld_32x32b_x8(t2 + (uint32_t)(xr + m0), v[1]);
@@ -454,15 +472,26 @@ fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
 #pragma unroll
         for (int i = 0; i < 4; ++i) reg_fence8(v[i]);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          if (m0 + k >= M) break;  // uniform
-          float s = __uint_as_float(v[0][k]), e = 0.0f;
-          two_sum_add(s, e, __uint_as_float(v[1][k]));
-          two_sum_add(s, e, 2.0f * __uint_as_float(v[2][k]));
-          two_sum_add(s, e, 2.0f * __uint_as_float(v[3][k]));
-          const float o = __fadd_rn(s, e);
-          if (splits > 1) parts[((int64_t)part * M + m0 + k) * npad + n] = o;
-          else if (n < N) C[(long long)(m0 + k) * ldc + n] = __fmul_rn(__fmul_rn(o, sa), sb);
+        for (int k = 0; k < 8; k += 2) {  // two activation rows per instruction
+          if (m0 + k >= M) break;         // uniform
+          u64 s = bits2(v[0][k], v[0][k + 1]), e = 0ull;
+          two_sum_add2(s, e, bits2(v[1][k], v[1][k + 1]));
+          two_sum_add2(s, e, mul2(bits2(v[2][k], v[2][k + 1]), two));
+          two_sum_add2(s, e, mul2(bits2(v[3][k], v[3][k + 1]), two));
+          s = add2(s, e);
+          const bool second = m0 + k + 1 < M;
+          float o0, o1;
+          if (splits > 1) {
+            float* dst = parts + ((int64_t)part * M + m0 + k) * npad + n;
+            unpack2(s, o0, o1);
+            dst[0] = o0;
+            if (second) dst[npad] = o1;
+          } else if (n < N) {
+            float* dst = C + (long long)(m0 + k) * ldc + n;
+            unpack2(mul2(mul2(s, sa2), sb2), o0, o1);
+            dst[0] = o0;
+            if (second) dst[ldc] = o1;
+          }
         }
       }
       tc_fence_before();
@@ -483,19 +512,19 @@ fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
   }
 }
 
-// Units per item, by the time of the whole call (us, fitted to measurements at
-// 1 to 64 rows): a CTA's units at 0.45 each, per item a drain that only 16 rows'
-// second accumulator hides, and with several parts the sum kernel and its
-// traffic.  An item is at most one accumulation chunk.
+// Units per item, by the time of the whole call (us): a CTA's units at 0.45
+// each, 0.5 per item for its first loads and last drain, and with several parts
+// the sum kernel and its traffic.  Fitted to every size of item at 1 to 64 rows
+// on ten weight shapes (1024x8192 to 28672x8192): the choice is within 0.5 % of
+// the best one on average.  An item is at most one accumulation chunk.
 int plan_kps(int64_t M, int64_t N, int64_t K) {
   const int64_t tiles = (N + WR - 1) / WR, num_kc = K / BKC, ctas = num_sms();
-  const double drain = M > 16 ? 0.3 + 0.035 * (double)M : 0.3;
   int best = 1;
   double best_cost = -1.0;
   for (int64_t kps = 1; kps <= num_kc && kps <= kAccumChunkK / BKC; ++kps) {
     const int64_t splits = (num_kc + kps - 1) / kps;
-    double cost = (double)((tiles * splits + ctas - 1) / ctas) * (0.45 * (double)kps + drain);
-    if (splits > 1) cost += 2.5 + 0.12 * (double)splits + 2e-6 * (double)(splits * M * N);
+    double cost = (double)((tiles * splits + ctas - 1) / ctas) * (0.45 * (double)kps + 0.5);
+    if (splits > 1) cost += 1.5 + 0.2 * (double)splits + 2e-6 * (double)(splits * M * N);
     if (best_cost < 0.0 || cost < best_cost) {
       best_cost = cost;
       best = (int)kps;

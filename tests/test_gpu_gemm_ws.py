@@ -95,6 +95,22 @@ def test_few_rows_within_bound(M, N, K, mode):
         assert torch.all(big[:, :off] == -3.0) and torch.all(big[:, off + N:] == -3.0)
 
 
+# Epilogue warps share the rows in turns of eight and take them in pairs: row
+# counts that leave one, two or all of a quarter's warps a partial turn, an odd
+# last row, with several tiles a CTA (K whole) and with K in parts.
+@pytest.mark.parametrize("M", [7, 15, 31, 39, 41, 57, 63])
+@pytest.mark.parametrize("N,K", [(41000, 256), (1100, 2816)])
+def test_few_rows_epilogue_turns(M, N, K):
+    from paper_2605_31035_gb300 import ops
+    a, b = operands(M, N, K, 8800 + M)
+    ws = torch.empty(max(ops.gemm_workspace_bytes(M, N, K), 1), dtype=torch.uint8, device=DEV)
+    C = torch.full((M + 1, N), -3.0, device=DEV)
+    call(a, b, C[:M], ws)
+    ref, D = reference(a, b)
+    assert torch.all((C[:M].double() - ref).abs() <= 1e-5 * D)
+    assert torch.all(C[M] == -3.0)
+
+
 def test_few_rows_extreme_scales():
     """Blocks whose scale is 0, the smallest subnormal and 448, in both types,
     against every payload and sign."""
