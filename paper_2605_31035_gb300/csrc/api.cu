@@ -56,7 +56,6 @@ int mixfp4_quantize(const void* x, int dtype, int64_t rows, int64_t K, int64_t l
   const uint16_t* xb = static_cast<const uint16_t*>(x);
   if (!given) {
     if (mixfp4::launch_quantize_small(xb, rows, K, ldx, codes, scales, tensor_scale, mode, s)) return launch_status();
-    if (cudaMemsetAsync(workspace, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
     mixfp4::launch_amax(xb, rows, K, ldx, workspace, s);
     if (int st = launch_status()) return st;
   }
@@ -86,7 +85,6 @@ int mixfp4_quantize_rht(const void* x, int dtype, int64_t rows, int64_t K, int64
   }
   const uint16_t* xb = static_cast<const uint16_t*>(x);
   if (!given) {
-    if (cudaMemsetAsync(workspace, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
     mixfp4::launch_rht_amax(xb, rows, K, ldx, signs, workspace, s);
     if (int st = launch_status()) return st;
   }
@@ -118,7 +116,6 @@ int quantize_colwise_impl(const void* x, int dtype, int64_t R, int64_t C, int64_
   }
   const uint16_t* xb = static_cast<const uint16_t*>(x);
   if (!given) {
-    if (cudaMemsetAsync(workspace, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
     mixfp4::launch_amax(xb, R, C, ldx, workspace, s);  // max |x| does not depend on the orientation
     if (int st = launch_status()) return st;
   }
@@ -165,7 +162,6 @@ int mixfp4_quantize_sr(const void* x, int dtype, int64_t rows, int64_t K, int64_
   }
   const uint16_t* xb = static_cast<const uint16_t*>(x);
   if (!given) {
-    if (cudaMemsetAsync(workspace, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
     mixfp4::launch_amax(xb, rows, K, ldx, workspace, s);
     if (int st = launch_status()) return st;
   }
@@ -196,7 +192,6 @@ int mixfp4_quantize_colwise_rht(const void* x, int dtype, int64_t R, int64_t C, 
   }
   const uint16_t* xb = static_cast<const uint16_t*>(x);
   if (!given) {
-    if (cudaMemsetAsync(workspace, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
     if (mixfp4::launch_quantize_colwise_rht(xb, R, C, ldx, signs, codes, scales, tensor_scale, workspace, mode, 0, 1,
                                             s) != 0)
       return MIXFP4_ERR_CUDA;
@@ -228,7 +223,6 @@ int mixfp4_quantize_2d(const void* x, int dtype, int64_t rows, int64_t K, int64_
   }
   const uint16_t* xb = static_cast<const uint16_t*>(x);
   if (!given) {
-    if (cudaMemsetAsync(workspace, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
     mixfp4::launch_amax(xb, rows, K, ldx, workspace, s);
     if (int st = launch_status()) return st;
   }
@@ -261,7 +255,6 @@ int mixfp4_fake_quantize(const void* x, int dtype, int64_t rows, int64_t K, int6
   }
   const uint16_t* xb = static_cast<const uint16_t*>(x);
   if (!given) {
-    if (cudaMemsetAsync(workspace, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
     mixfp4::launch_amax(xb, rows, K, ldx, workspace, s);
     if (int st = launch_status()) return st;
   }

@@ -116,7 +116,6 @@ extern "C" int mixfp4_quantize_noalloc(const void* x, int dtype, int64_t rows, i
   }
   uint32_t* amax_word = scratch_for_current_device();
   if (!amax_word) return MIXFP4_ERR_CUDA;
-  if (cudaMemsetAsync(amax_word, 0, kAmaxWords * sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
   const uint16_t* xb = static_cast<const uint16_t*>(x);
   mixfp4::launch_amax(xb, rows, K, ldx, amax_word, s);
   if (cudaGetLastError() != cudaSuccess) return MIXFP4_ERR_CUDA;

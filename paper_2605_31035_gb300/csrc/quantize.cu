@@ -311,6 +311,7 @@ rht_amax_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = max(m, red[i]);
+    griddep_wait();  // the word is zeroed by then
     if (m) atomicMax(amax_word, m);
   }
   griddep_launch_dependents();
@@ -318,8 +319,24 @@ rht_amax_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks
 
 // max |x| over the tensor as the bit pattern of a non-negative fp32 (bf16
 // magnitudes order like unsigned 16-bit integers).  Each thread keeps four
-// 32-byte loads in flight.
-constexpr int kAmaxUnroll = 4;
+// 32-byte loads in flight: a register set is loaded again as soon as it has been
+// looked at (a set past the end keeps its old values, which change no maximum).
+// The tensor is read from its end: the pass that follows starts at the front and
+// finds what was read last in L2 (both passes of 8192 x 8192: 69.6 us forward,
+// 63.3; 65536 x 4096: 254, 245; no gain for the rotated passes, which arithmetic
+// bounds).  Three CTAs per SM of this loop against eight of batches of four
+// loads, with the kernel below in place of the memset: 4096 x 4096 21.1 -> 17.6,
+// 1024 x 4096 10.4 -> 7.4.  Four CTAs per SM: 18.4 (spills); two: 17.5 and 64.4.
+constexpr int kAmaxUnroll = 4, kAmaxCtas = 3;
+
+// The word is zeroed once everything before is complete; the dependents (the
+// maximum passes) therefore read their tensor without waiting, and wait only
+// before they touch the word.  As a memset it and its gaps cost 3.3 us a call.
+__global__ void zero_word_kernel(uint32_t* word) {
+  griddep_wait();
+  griddep_launch_dependents();
+  if (threadIdx.x == 0) *word = 0u;
+}
 
 template <bool kContig>
 __device__ __forceinline__ const uint16_t* amax_src(const uint16_t* x, int64_t b, int64_t kblocks, int64_t ldx) {
@@ -332,27 +349,28 @@ __device__ __forceinline__ const uint16_t* amax_src(const uint16_t* x, int64_t b
 // kernel to reduce, so nothing has to be zeroed first (a memset and its gaps
 // are about 2.5 us of a call).
 template <bool kContig, bool kParts>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, kAmaxCtas)
 amax_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, int64_t ldx,
             uint32_t* amax_word) {
   if (kParts) griddep_wait();
   uint32_t m = 0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nblocks; b += kAmaxUnroll * stride) {
-    uint32_t w[kAmaxUnroll][8];
+  int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  uint32_t w[kAmaxUnroll][8];
+#pragma unroll
+  for (int u = 0; u < kAmaxUnroll; ++u) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w[u][j] = 0u;
+    if (b + u * stride < nblocks) ldg256_stream(amax_src<kContig>(x, nblocks - 1 - b - u * stride, kblocks, ldx), w[u]);
+  }
+  for (; b < nblocks; b += kAmaxUnroll * stride)
 #pragma unroll
     for (int u = 0; u < kAmaxUnroll; ++u) {
-      const int64_t bu = b + u * stride;
-      if (bu < nblocks) ldg256_stream(amax_src<kContig>(x, bu, kblocks, ldx), w[u]);
-      else
-#pragma unroll
-        for (int j = 0; j < 8; ++j) w[u][j] = 0u;
-    }
-#pragma unroll
-    for (int u = 0; u < kAmaxUnroll; ++u)
 #pragma unroll
       for (int j = 0; j < 8; ++j) m = __vmaxu2(m, w[u][j] & 0x7FFF7FFFu);
-  }
+      const int64_t next = b + (kAmaxUnroll + u) * stride;
+      if (next < nblocks) ldg256_stream(amax_src<kContig>(x, nblocks - 1 - next, kblocks, ldx), w[u]);
+    }
   m = max(m & 0xFFFFu, m >> 16);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -361,8 +379,12 @@ amax_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, in
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = max(m, red[i]);
-    if (kParts) amax_word[blockIdx.x] = m << 16;
-    else if (m) atomicMax(amax_word, m << 16);
+    if (kParts) {
+      amax_word[blockIdx.x] = m << 16;
+    } else {
+      griddep_wait();  // the word is zeroed by then
+      if (m) atomicMax(amax_word, m << 16);
+    }
   }
   // The quantize kernel that follows may start once every CTA got here.
   griddep_launch_dependents();
@@ -403,14 +425,30 @@ dequantize_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__
 
 }  // namespace
 
+// Zero the word a maximum is taken into, by a kernel instead of a memset: the
+// pass over the tensor is its programmatic dependent and overlaps it.
+int launch_zero_word(uint32_t* word, cudaStream_t stream) {
+  return launch_pdl(zero_word_kernel, 1, 32, 0, stream, word) == cudaSuccess ? 0 : -1;
+}
+
+// The resident CTAs, or, above 2^23 blocks (268 MB), more than fit at once: over
+// such a length the CTAs drift apart and the late ones end alone (tensor out of
+// L2, both passes: 65536 x 4096 267 us against 263; 32768 x 4096 140 both ways;
+// 8192 x 4096 42 against 44).
+static int64_t amax_grid(int64_t nblocks) {
+  const int64_t grid = (nblocks + 256 * kAmaxUnroll - 1) / (256 * kAmaxUnroll);
+  const int64_t cap = num_sms() * (nblocks > (1 << 23) ? 8 : kAmaxCtas);
+  return grid < cap ? grid : cap;
+}
+
 int launch_amax(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint32_t* amax_word,
                 cudaStream_t stream) {
   const int64_t kblocks = K / 16, nblocks = rows * kblocks;
   if (nblocks == 0) return 0;
-  int64_t grid = (nblocks + 256 * kAmaxUnroll - 1) / (256 * kAmaxUnroll);
-  if (grid > num_sms() * 8) grid = num_sms() * 8;
-  if (ldx == K) amax_kernel<true, false><<<(unsigned)grid, 256, 0, stream>>>(x, nblocks, kblocks, ldx, amax_word);
-  else amax_kernel<false, false><<<(unsigned)grid, 256, 0, stream>>>(x, nblocks, kblocks, ldx, amax_word);
+  launch_zero_word(amax_word, stream);
+  const unsigned grid = (unsigned)amax_grid(nblocks);
+  if (ldx == K) launch_pdl(amax_kernel<true, false>, grid, 256, 0, stream, x, nblocks, kblocks, ldx, amax_word);
+  else launch_pdl(amax_kernel<false, false>, grid, 256, 0, stream, x, nblocks, kblocks, ldx, amax_word);
   return 0;
 }
 
@@ -418,8 +456,7 @@ int launch_amax(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint32_
 static void launch_amax_parts(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint32_t* parts, int* n,
                               cudaStream_t stream) {
   const int64_t kblocks = K / 16, nblocks = rows * kblocks;
-  int64_t grid = (nblocks + 256 * kAmaxUnroll - 1) / (256 * kAmaxUnroll);
-  if (grid > num_sms() * 8) grid = num_sms() * 8;
+  int64_t grid = amax_grid(nblocks);
   if (grid > kMaxAmaxParts) grid = kMaxAmaxParts;
   *n = (int)grid;
   if (ldx == K) launch_pdl(amax_kernel<true, true>, (unsigned)grid, 256, 0, stream, x, nblocks, kblocks, ldx, parts);
@@ -522,8 +559,9 @@ int launch_rht_amax(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, con
   if (nblocks == 0) return 0;
   int64_t grid = (nblocks + 255) / 256;
   if (grid > num_sms() * 8) grid = num_sms() * 8;
-  if (ldx == K) rht_amax_kernel<true><<<(unsigned)grid, 256, 0, stream>>>(x, nblocks, kblocks, ldx, signs, amax_word);
-  else rht_amax_kernel<false><<<(unsigned)grid, 256, 0, stream>>>(x, nblocks, kblocks, ldx, signs, amax_word);
+  launch_zero_word(amax_word, stream);
+  if (ldx == K) launch_pdl(rht_amax_kernel<true>, (unsigned)grid, 256, 0, stream, x, nblocks, kblocks, ldx, signs, amax_word);
+  else launch_pdl(rht_amax_kernel<false>, (unsigned)grid, 256, 0, stream, x, nblocks, kblocks, ldx, signs, amax_word);
   return 0;
 }
 

@@ -255,7 +255,7 @@ quantize_colwise_rht_kernel(const uint16_t* __restrict__ x, int64_t R, int64_t C
                             uint8_t* __restrict__ scales, float* tensor_scale, uint32_t* amax_word, int scale_given) {
   __shared__ float4 tab[128];
   __shared__ __align__(16) float tiles_s[kCrWarps][kCrTile];
-  griddep_wait();
+  if (!kAmax) griddep_wait();  // the maximum pass follows launch_zero_word, which waits for all before
   griddep_launch_dependents();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int cp = lane & 7, g = lane >> 3;  // column pair, and which of four blocks / residues
@@ -354,6 +354,7 @@ quantize_colwise_rht_kernel(const uint16_t* __restrict__ x, int64_t R, int64_t C
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int i = 1; i < kCrWarps; ++i) m = max(m, red[i]);
+      griddep_wait();  // the word is zeroed by then
       if (m) atomicMax(amax_word, m);
     }
   }
@@ -538,6 +539,7 @@ int launch_quantize_colwise_rht(const uint16_t* x, int64_t R, int64_t C, int64_t
   e = launch_pdl(quantize_colwise_rht_kernel<MODE, AMAX>, (unsigned)grid, 32 * kCrWarps, 0, stream, x, R, C, ldx, signs, \
                  codes, scales, tensor_scale, amax_word, scale_given)
   if (amax_pass) {
+    if (launch_zero_word(amax_word, stream) != 0) return -1;
     MIXFP4_LAUNCH_CR(MIXFP4_MODE_MIX, true);
   } else {
     switch (mode) {
