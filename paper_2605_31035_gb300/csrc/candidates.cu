@@ -202,9 +202,9 @@ fake_quantize_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t K, in
                      float* tensor_scale, const uint32_t* amax_word, int scale_given, void* __restrict__ out,
                      int out_bf16, int64_t ldo, uint8_t* __restrict__ choice) {
   __shared__ float4 tab[128];  // E4M3 code -> {s8, zh, zl, 0}
+  fill_scale_table(tab);
   griddep_wait();
   griddep_launch_dependents();
-  fill_scale_table(tab);
   const TensorConsts tc = tensor_consts(tensor_scale, amax_word, scale_given);
   const bool markstein = markstein_needed(tc);  // ends with a CTA barrier (tab is ready)
   const float s32 = tc.scaled ? scalbnf(tc.s32, -tc.k) : tc.s32;  // the tensor's own s32 (exact)

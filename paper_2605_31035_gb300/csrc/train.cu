@@ -49,9 +49,9 @@ quantize_colwise_kernel(const uint16_t* __restrict__ x, int64_t R, int64_t C, in
   // Row pairs interleaved: pairs[p][c] = x[2p][c] | x[2p + 1][c] << 16, the
   // bf16 pair of column c that quantize_block takes as one word.
   __shared__ __align__(16) uint32_t pairs[kColRows / 2][kColThreads];
+  fill_scale_table(tab);  // under the kernel before; with it 1024 x 4096 takes 0.3 to 0.5 us less
   griddep_wait();
   griddep_launch_dependents();
-  fill_scale_table(tab);
   const TensorConsts tc = tensor_consts(tensor_scale, amax_word, scale_given);
   const bool markstein = markstein_needed(tc);
   const int tid = threadIdx.x;
@@ -159,9 +159,9 @@ quantize_sr_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblo
                    uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, float* tensor_scale,
                    const uint32_t* amax_word, int scale_given, uint64_t seed, uint64_t offset) {
   __shared__ float4 tab[128];
+  fill_scale_table(tab);
   griddep_wait();
   griddep_launch_dependents();
-  fill_scale_table(tab);
   const TensorConsts tc = tensor_consts(tensor_scale, amax_word, scale_given);
   const bool markstein = markstein_needed(tc);
   const int64_t nthr = (int64_t)gridDim.x * blockDim.x;
@@ -179,9 +179,9 @@ quantize_2d_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t K, int6
                    uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, float* tensor_scale,
                    const uint32_t* amax_word, int scale_given) {
   __shared__ float4 tab[128];
+  fill_scale_table(tab);
   griddep_wait();
   griddep_launch_dependents();
-  fill_scale_table(tab);
   const TensorConsts tc = tensor_consts(tensor_scale, amax_word, scale_given);
   const bool markstein = markstein_needed(tc);
   const int lane = threadIdx.x & 31, i = lane & 15, h = lane >> 4;
@@ -255,7 +255,10 @@ quantize_colwise_rht_kernel(const uint16_t* __restrict__ x, int64_t R, int64_t C
                             uint8_t* __restrict__ scales, float* tensor_scale, uint32_t* amax_word, int scale_given) {
   __shared__ float4 tab[128];
   __shared__ __align__(16) float tiles_s[kCrWarps][kCrTile];
-  if (!kAmax) griddep_wait();  // the maximum pass follows launch_zero_word, which waits for all before
+  if (!kAmax) {  // the maximum pass follows launch_zero_word, which waits for all before
+    fill_scale_table(tab);
+    griddep_wait();
+  }
   griddep_launch_dependents();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int cp = lane & 7, g = lane >> 3;  // column pair, and which of four blocks / residues
@@ -267,7 +270,6 @@ quantize_colwise_rht_kernel(const uint16_t* __restrict__ x, int64_t R, int64_t C
       bits[h] = (uint32_t)__ldg(signs + 2 * (g + 4 * h)) | ((uint32_t)__ldg(signs + 2 * (g + 4 * h) + 1) << 8);
   TensorConsts tc{};
   if (!kAmax) {
-    fill_scale_table(tab);
     tc = tensor_consts(tensor_scale, amax_word, scale_given);
     __syncthreads();
   }
