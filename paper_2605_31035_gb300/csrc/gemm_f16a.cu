@@ -148,7 +148,7 @@ gemm_f16a_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
                  const __grid_constant__ CUtensorMap tm_bs, const __grid_constant__ CUtensorMap tm_c, int c_tma,
                  const float* __restrict__ a_ts, const float* __restrict__ b_ts, int M, int N, int K,
                  float* __restrict__ C, long long ldc, int tile_n, int dp_tiles, int chunk_kc, int splits, int kps,
-                 uint32_t* status_word) {
+                 int after_zero, uint32_t* status_word) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   Bars* bars = reinterpret_cast<Bars*>(smem + OFF_BAR);
@@ -202,7 +202,7 @@ gemm_f16a_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     // ---------------- TMA producer: A ----------------
     if (elect_one()) {
       tma_prefetch(&tm_a);
-      griddep_wait();
+      if (!after_zero) griddep_wait();  // launch_zero_rows has waited for the operands
       int it = 0, last = -1;
       bool ok = true;
       while (ok && work.next(t, k0, k1)) {
@@ -272,7 +272,7 @@ gemm_f16a_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     if (elect_one()) {
       tma_prefetch(&tm_bc);
       tma_prefetch(&tm_bs);
-      griddep_wait();
+      if (!after_zero) griddep_wait();
       const uint32_t tx = (uint32_t)b_rows * (BKC / 2 + BKC / 16);
       int it = 0, last = -1;
       bool ok = true;
@@ -628,15 +628,11 @@ int launch_gemm_f16a(const void* a_f16, const float* a_ts, const uint8_t* b_code
     // Zero C from the first split tile's row band down (whole tiles among those
     // rows are overwritten by plain stores after this).
     const int64_t r0 = (p.dp_tiles / ntiles_n) * fa::TILE_M;
-    const cudaError_t e =
-        ldc == N ? cudaMemsetAsync(C + r0 * ldc, 0, (size_t)(M - r0) * (size_t)N * sizeof(float), stream)
-                 : cudaMemset2DAsync(C + r0 * ldc, (size_t)ldc * sizeof(float), 0, (size_t)N * sizeof(float),
-                                     (size_t)(M - r0), stream);
-    if (e != cudaSuccess) return MIXFP4_ERR_CUDA;
+    if (launch_zero_rows(C + r0 * ldc, M - r0, N, ldc, stream) != 0) return MIXFP4_ERR_CUDA;
   }
   if (launch_pdl(fa::gemm_f16a_kernel, (unsigned)(2 * clusters), fa::kThreads, fa::SMEM_ALLOC, stream, ta, tbc, tbs,
                  tmc, c_tma, a_ts, b_ts, (int)M, (int)N, (int)K, C, (long long)ldc, p.tile_n, (int)p.dp_tiles,
-                 kAccumChunkK / fa::BKC, p.splits, p.kps, status_word) != cudaSuccess)
+                 kAccumChunkK / fa::BKC, p.splits, p.kps, p.dp_tiles < p.tiles ? 1 : 0, status_word) != cudaSuccess)
     return MIXFP4_ERR_CUDA;
   if (p.splits > 1)
     return launch_sum_parts(static_cast<const float*>(parts), p.splits, m_pad * ldp, ldp, 0.25f, a_ts, b_ts, M, N, C,

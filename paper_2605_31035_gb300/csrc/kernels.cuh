@@ -9,6 +9,7 @@
 namespace mixfp4 {
 
 int launch_zero_word(uint32_t* word, cudaStream_t stream);
+int launch_zero_rows(float* C, int64_t rows, int64_t cols, int64_t ldc, cudaStream_t stream);
 int launch_amax(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint32_t* amax_word,
                 cudaStream_t stream);
 int launch_quantize(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, uint8_t* codes,

@@ -87,6 +87,8 @@ __global__ void __launch_bounds__(256) split_native_kernel(const uint8_t* __rest
                                                            int64_t K, uint8_t* __restrict__ main_codes,
                                                            uint8_t* __restrict__ res_codes, uint8_t* __restrict__ sf,
                                                            int64_t n_code, int64_t n_sf) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int64_t nb = K / 16;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_code + n_sf;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -179,7 +181,7 @@ nvf4_gemm_kernel(const __grid_constant__ CUtensorMap tm_am, const __grid_constan
                  const __grid_constant__ CUtensorMap tm_bm, const __grid_constant__ CUtensorMap tm_br,
                  const uint8_t* __restrict__ a_sf, const uint8_t* __restrict__ b_sf, const float* __restrict__ a_ts,
                  const float* __restrict__ b_ts, int M, int N, int K, float* __restrict__ C, long long ldc,
-                 int dp_tiles, int chunk_kc, uint32_t* status_word) {
+                 int dp_tiles, int chunk_kc, int after_zero, uint32_t* status_word) {
   using L = Layout<kARes, kBRes>;
   constexpr int S = L::kStages;
   extern __shared__ uint8_t smem_raw[];
@@ -230,7 +232,7 @@ nvf4_gemm_kernel(const __grid_constant__ CUtensorMap tm_am, const __grid_constan
       tma_prefetch(&tm_bm);
       if (kARes) tma_prefetch(&tm_ar);
       if (kBRes) tma_prefetch(&tm_br);
-      griddep_wait();
+      if (!after_zero) griddep_wait();  // launch_zero_rows has waited for the operands
       int last_it = -1, it = 0;
       bool ok = true;
       Sched sched(cluster_id, nclusters, dp_tiles, ntiles, num_kc, chunk_kc);
@@ -441,17 +443,11 @@ int launch(const uint8_t* a_main, const uint8_t* a_res, const uint8_t* a_sf, con
     dp_tiles = tiles - rem;
   if (dp_tiles < tiles) {
     const int64_t r0 = (dp_tiles / ntiles_n) * TILE_M;
-    cudaError_t e;
-    if (ldc == N)
-      e = cudaMemsetAsync(C + r0 * ldc, 0, (size_t)(M - r0) * (size_t)N * sizeof(float), stream);
-    else
-      e = cudaMemset2DAsync(C + r0 * ldc, (size_t)ldc * sizeof(float), 0, (size_t)N * sizeof(float),
-                            (size_t)(M - r0), stream);
-    if (e != cudaSuccess) return MIXFP4_ERR_CUDA;
+    if (launch_zero_rows(C + r0 * ldc, M - r0, N, ldc, stream) != 0) return MIXFP4_ERR_CUDA;
   }
   if (launch_pdl(nvf4_gemm_kernel<kARes, kBRes>, (unsigned)(2 * clusters), kThreads, L::SMEM_ALLOC, stream, tam,
                  tar, tbm, tbr, a_sf, b_sf, a_ts, b_ts, (int)M, (int)N, (int)K, C, (long long)ldc, (int)dp_tiles,
-                 kAccumChunkK / BKC, status_word) != cudaSuccess)
+                 kAccumChunkK / BKC, dp_tiles < tiles ? 1 : 0, status_word) != cudaSuccess)
     return MIXFP4_ERR_CUDA;
   return MIXFP4_OK;
 }
@@ -631,8 +627,7 @@ nvf4_fewrows_kernel(const __grid_constant__ CUtensorMap tm_wc, const __grid_cons
       tma_prefetch(&tm_wc);
       tma_prefetch(&tm_ws);
       tma_prefetch(&tm_xc);
-      tma_prefetch(&tm_xs);
-      griddep_wait();
+      tma_prefetch(&tm_xs);  // the operands are complete: launch_zero_rows has waited for them
       int it = 0;
       long long last = -1;
       for (long long u = u_begin; u < u_end; ++u, ++it) {
@@ -862,12 +857,7 @@ int launch(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts, c
   static std::atomic<uint64_t> smem_set{0};
   if (!set_dynamic_smem_once(reinterpret_cast<const void*>(nvf4_fewrows_kernel), 232448, smem_set))
     return MIXFP4_ERR_CUDA;
-  cudaError_t e;
-  if (ldc == N)
-    e = cudaMemsetAsync(C, 0, (size_t)M * (size_t)N * sizeof(float), stream);
-  else
-    e = cudaMemset2DAsync(C, (size_t)ldc * sizeof(float), 0, (size_t)N * sizeof(float), (size_t)M, stream);
-  if (e != cudaSuccess) return MIXFP4_ERR_CUDA;
+  if (launch_zero_rows(C, M, N, ldc, stream) != 0) return MIXFP4_ERR_CUDA;
   const int64_t units = ((N + WR - 1) / WR) * (K / BKC);
   int64_t grid = num_sms();
   if (grid > units) grid = units;
@@ -888,9 +878,10 @@ int launch_split_native(const uint8_t* codes, const uint8_t* scales, int64_t row
   int64_t blocks = (n_code + n_sf + 255) / 256;
   const int64_t cap = (int64_t)num_sms() * 8;
   if (blocks > cap) blocks = cap;
-  split_native_kernel<<<(unsigned)blocks, 256, 0, stream>>>(codes, scales, rows, K, main_codes, res_codes, sf, n_code,
-                                                            n_sf);
-  return cudaGetLastError() == cudaSuccess ? MIXFP4_OK : MIXFP4_ERR_CUDA;
+  return launch_pdl(split_native_kernel, (unsigned)blocks, 256, 0, stream, codes, scales, rows, K, main_codes, res_codes,
+                    sf, n_code, n_sf) == cudaSuccess
+             ? MIXFP4_OK
+             : MIXFP4_ERR_CUDA;
 }
 
 int launch_gemm_native(const uint8_t* a_main, const uint8_t* a_res, const uint8_t* a_sf, const float* a_ts,

@@ -317,6 +317,21 @@ rht_amax_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks
   }
 }
 
+__global__ void __launch_bounds__(256)
+zero_rows_kernel(float* __restrict__ C, int64_t n, int64_t per_row, int64_t cols, int64_t ldc, int vec) {
+  griddep_wait();
+  griddep_launch_dependents();
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = i / per_row, c = (i - r * per_row) * (vec ? 4 : 1);
+    float* dst = C + r * ldc + c;
+    if (vec && c + 4 <= cols) {
+      *reinterpret_cast<float4*>(dst) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    } else {
+      for (int64_t k = 0; k < (vec ? cols - c : 1); ++k) dst[k] = 0.0f;
+    }
+  }
+}
+
 // max |x| over the tensor as the bit pattern of a non-negative fp32 (bf16
 // magnitudes order like unsigned 16-bit integers).  Each thread keeps four
 // 32-byte loads in flight: a register set is loaded again as soon as it has been
@@ -431,6 +446,25 @@ dequantize_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__
 // pass over the tensor is its programmatic dependent and overlaps it.
 int launch_zero_word(uint32_t* word, cudaStream_t stream) {
   return launch_pdl(zero_word_kernel, 1, 32, 0, stream, word) == cudaSuccess ? 0 : -1;
+}
+
+// Zero `rows` rows of `cols` floats (row stride ldc), for a GEMM that adds parts
+// into them.  Like launch_zero_word it waits for all before, so the GEMM (its
+// programmatic dependent) may load its operands meanwhile and waits only before it
+// touches C.  Against a memset: native GEMM 1536 x 4096 x 4096 47.2 -> 45.1 us, 4096^3
+// 86.2 -> 81.9, GEMM with A decoded beforehand 2560 x 4096 x 4096 59.6 -> 57.4.
+int launch_zero_rows(float* C, int64_t rows, int64_t cols, int64_t ldc, cudaStream_t stream) {
+  if (ldc == cols) {  // one long row
+    cols *= rows;
+    rows = 1;
+  }
+  const bool vec = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && (rows == 1 || (ldc & 3) == 0);
+  const int64_t per_row = vec ? (cols + 3) / 4 : cols, n = rows * per_row;
+  int64_t grid = (n + 255) / 256;
+  if (grid > num_sms() * 4) grid = num_sms() * 4;
+  return launch_pdl(zero_rows_kernel, (unsigned)grid, 256, 0, stream, C, n, per_row, cols, ldc, vec ? 1 : 0) == cudaSuccess
+             ? 0
+             : -1;
 }
 
 // The resident CTAs, or, above 2^23 blocks (268 MB), more than fit at once: over
