@@ -156,6 +156,7 @@ quantize_small_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t k
                       uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, float* tensor_scale, int xr) {
   __shared__ float4 tab[128];
   __shared__ uint32_t red[kSmallThreads / 32], maxes[kSmallCtas], amax;
+  sm100::cluster_arrive();  // awaited before the first store into another CTA
   griddep_wait();
   griddep_launch_dependents();
   const int64_t b0 = (int64_t)blockIdx.x * kSmallThreads + threadIdx.x;
@@ -178,6 +179,9 @@ quantize_small_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t k
   m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
+  // The CTAs of a cluster are scheduled together, but only a cluster barrier says
+  // that the others have started; a store into one that has not is undefined.
+  sm100::cluster_wait();
   if (threadIdx.x < 32) {
     m = __reduce_max_sync(0xffffffffu, threadIdx.x < kSmallThreads / 32 ? red[threadIdx.x] : 0u);
     if (threadIdx.x < kSmallCtas)

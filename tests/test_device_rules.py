@@ -1,0 +1,48 @@
+"""Rules of the CUDA sources that a run cannot show to be broken (it works until
+the scheduling changes), checked by reading the kernels on CPU."""
+import os
+import re
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2605_31035_gb300", "csrc")
+
+
+def strip_comments(text):
+    return re.sub(r"//[^\n]*|/\*.*?\*/", "", text, flags=re.S)
+
+
+def kernels():
+    """(file, name, parameters, body) of every __global__ function."""
+    out = []
+    for f in sorted(os.listdir(CSRC)):
+        text = strip_comments(open(os.path.join(CSRC, f)).read())
+        for m in re.finditer(r"__global__[^;{]*?\b(\w+_kernel)\s*\(([^{]*)\)\s*\{", text):
+            depth, i = 1, m.end()
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[i], 0)
+                i += 1
+            out.append((f, m.group(1), m.group(2), text[m.end():i]))
+    return out
+
+
+KERNELS = kernels()
+
+
+def test_every_kernel_is_found():
+    launches = sum(len(re.findall(r"__global__", strip_comments(open(os.path.join(CSRC, f)).read())))
+                   for f in os.listdir(CSRC))
+    assert len(KERNELS) == launches > 20
+
+
+# CUDA defines accesses to another CTA's shared memory only once that CTA has
+# started, which a barrier of the whole cluster is the way to know.
+REMOTE = [k for k in KERNELS if re.search(r"mapa_shared|st_cluster", k[3])]
+
+
+@pytest.mark.parametrize("name,body", [(k[1], k[3]) for k in REMOTE], ids=[k[1] for k in REMOTE])
+def test_cluster_barrier_before_remote_shared_memory(name, body):
+    barrier = re.search(r"\bcluster_(sync|wait)\s*\(\s*\)", body)
+    remote = re.search(r"\bst_cluster_\w+\s*\(|\bmbar_arrive_cluster\s*\(|\bmma_commit_pair\s*\(", body)
+    assert barrier and remote and barrier.start() < remote.start(), name
