@@ -198,7 +198,7 @@ __device__ __forceinline__ void fake_quantize_unit(const u64 a[8], const TensorC
 // kDense: rows of x and out follow one another without gaps.
 template <int kG, bool kDense>
 __global__ void __launch_bounds__(kFqThreads, 4)
-fake_quantize_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t K, int64_t ldx, int mask,
+fake_quantize_kernel(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx, int mask,
                      float* tensor_scale, const uint32_t* amax_word, int scale_given, void* __restrict__ out,
                      int out_bf16, int64_t ldo, uint8_t* __restrict__ choice) {
   __shared__ float4 tab[128];  // E4M3 code -> {s8, zh, zl, 0}

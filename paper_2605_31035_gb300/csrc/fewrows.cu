@@ -147,8 +147,8 @@ static_assert(sizeof(Bars) <= OFF_RINGS, "barrier block");
 
 // Activation operand: thread = 16-byte chunk (32 codes) of one of XR rows.
 __global__ void __launch_bounds__(256)
-fewrows_prep_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales, int M, int xr, int K,
-                    uint8_t* __restrict__ xop, uint8_t* __restrict__ sfa) {
+fewrows_prep_kernel(const uint8_t* codes, const uint8_t* scales, int M, int xr, int K, uint8_t* __restrict__ xop,
+                    uint8_t* __restrict__ sfa) {
   griddep_wait();
   griddep_launch_dependents();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -158,8 +158,8 @@ fewrows_prep_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict
   uint4 w = make_uint4(0u, 0u, 0u, 0u);
   uint32_t s4 = 0u;  // scales of the 64-K step this chunk lies in
   if (r < M) {
-    w = __ldg(reinterpret_cast<const uint4*>(codes + (int64_t)r * (K / 2)) + c);
-    s4 = __ldg(reinterpret_cast<const uint32_t*>(scales + (int64_t)r * (K / 16)) + c / 2);
+    w = reinterpret_cast<const uint4*>(codes + (int64_t)r * (K / 2))[c];
+    s4 = reinterpret_cast<const uint32_t*>(scales + (int64_t)r * (K / 16))[c / 2];
   }
   const uint32_t m0 = type_mask(s4, 2 * (c & 1)), m1 = type_mask(s4, 2 * (c & 1) + 1);
   const uint4 q = make_uint4(residual_word(w.x) & m0, residual_word(w.y) & m0, residual_word(w.z) & m1,
@@ -184,9 +184,9 @@ constexpr int kAhead = 2;
 
 __global__ void __launch_bounds__(kThreads, 1)
 fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
-               const uint8_t* __restrict__ w_scales, const uint8_t* __restrict__ sfa, int M, int xr, int N, int K,
-               int splits, int kps, const float* __restrict__ a_ts, const float* __restrict__ b_ts,
-               float* __restrict__ parts, float* __restrict__ C, long long ldc, uint32_t* status_word) {
+               const uint8_t* w_scales, const uint8_t* sfa, int M, int xr, int N, int K, int splits, int kps,
+               const float* a_ts, const float* b_ts, float* __restrict__ parts, float* __restrict__ C, long long ldc,
+               uint32_t* status_word) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   Bars* bars = reinterpret_cast<Bars*>(smem);
@@ -445,7 +445,7 @@ fewrows_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
     // D2 and D1 are activation row m's main and residual products.
     const int q = warp & 3;
     griddep_wait();
-    const float sa = __ldg(a_ts), sb = __ldg(b_ts);
+    const float sa = a_ts[0], sb = b_ts[0];
     const u64 sa2 = pack2(sa, sa), sb2 = pack2(sb, sb), two = pack2(2.0f, 2.0f);
     const int npad = tiles * WR;
     const int set = warp < kFirstSplit ? 0 : (warp - kFirstSplit) / 4 - 2 * groups(xr) + 1;

@@ -161,7 +161,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairRoles<kTileN>::k
 mixfp4_gemm_kernel(const __grid_constant__ CUtensorMap tm_ac, const __grid_constant__ CUtensorMap tm_bc,
                    const __grid_constant__ CUtensorMap tm_as, const __grid_constant__ CUtensorMap tm_bs,
                    const __grid_constant__ CUtensorMap tm_c, int c_tma,
-                   const float* __restrict__ a_ts, const float* __restrict__ b_ts,
+                   const float* a_ts, const float* b_ts,
                    int M, int N, int K, float* __restrict__ C, long long ldc, int dp_tiles, int chunk_kc,
                    uint32_t* status_word, uint64_t wait_ns, int skip_first_stage) {
   extern __shared__ uint8_t smem_raw[];
@@ -414,7 +414,7 @@ mixfp4_gemm_kernel(const __grid_constant__ CUtensorMap tm_ac, const __grid_const
     const int chalf = (warp - kFirstEpi) >> 2;  // column half
     const bool elected = elect_one();
     griddep_wait();
-    const float sa = 0.25f * __ldg(a_ts), sb = __ldg(b_ts);
+    const float sa = 0.25f * a_ts[0], sb = b_ts[0];
     const u64 sa2 = pack2(sa, sa), sb2 = pack2(sb, sb);
     const uint32_t acc_empty_leader = mapa_shared(smem_u32(&bars->acc_empty), 0);
     // Staging tiles: the warp's own, and for tiles of at most 224 columns a

@@ -58,13 +58,12 @@ using namespace sm100;
 // ------------------------------------------------------------ operand decode
 // Thread per 16-byte chunk (32 codes of one row): 16 + 2 bytes in, 64 out.
 __global__ void __launch_bounds__(256)
-decode_f16_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales, int64_t nchunks,
-                  uint8_t* __restrict__ out) {
+decode_f16_kernel(const uint8_t* codes, const uint8_t* scales, int64_t nchunks, uint8_t* __restrict__ out) {
   griddep_wait();
   griddep_launch_dependents();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nchunks; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint4 c = __ldg(reinterpret_cast<const uint4*>(codes) + i);
-    const uint32_t s = __ldg(reinterpret_cast<const uint16_t*>(scales) + i);
+    const uint4 c = reinterpret_cast<const uint4*>(codes)[i];
+    const uint32_t s = reinterpret_cast<const uint16_t*>(scales)[i];
     uint32_t o[16];
     decode_chunk(c, s, o);
     stg256(out + i * 64, o);
@@ -146,7 +145,7 @@ struct Work {
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 gemm_f16a_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_bc,
                  const __grid_constant__ CUtensorMap tm_bs, const __grid_constant__ CUtensorMap tm_c, int c_tma,
-                 const float* __restrict__ a_ts, const float* __restrict__ b_ts, int M, int N, int K,
+                 const float* a_ts, const float* b_ts, int M, int N, int K,
                  float* __restrict__ C, long long ldc, int tile_n, int dp_tiles, int chunk_kc, int splits, int kps,
                  int after_zero, uint32_t* status_word) {
   extern __shared__ uint8_t smem_raw[];
@@ -381,7 +380,7 @@ gemm_f16a_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     const bool elected = elect_one();
     griddep_wait();
     // Parts of a split K are stored unscaled: sum_parts_kernel scales their sum.
-    const float sa = splits > 1 ? 1.0f : 0.25f * __ldg(a_ts), sb = splits > 1 ? 1.0f : __ldg(b_ts);
+    const float sa = splits > 1 ? 1.0f : 0.25f * a_ts[0], sb = splits > 1 ? 1.0f : b_ts[0];
     const u64 sa2 = pack2(sa, sa), sb2 = pack2(sb, sb);
     const uint32_t acc_empty0 = mapa_shared(smem_u32(&bars->acc_empty[0]), 0);
     const uint32_t stage = sbase + OFF_EPI + (uint32_t)ew * EPI_BYTES;
@@ -464,12 +463,11 @@ gemm_f16a_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
 // (Knuth's two-sum), so splitting K costs no accuracy: on 100 x 512 x 14336 the
 // parts added into C one by one in fp32 left twice the error of one pass.
 __global__ void __launch_bounds__(256)
-sum_parts_kernel(const float* __restrict__ parts, int splits, long long part_stride, int ldp,
-                 float factor, const float* __restrict__ a_ts, const float* __restrict__ b_ts, int M, int N,
-                 float* __restrict__ C, long long ldc, int vec) {
+sum_parts_kernel(const float* parts, int splits, long long part_stride, int ldp, float factor, const float* a_ts,
+                 const float* b_ts, int M, int N, float* __restrict__ C, long long ldc, int vec) {
   griddep_wait();
   griddep_launch_dependents();
-  const float sa = factor * __ldg(a_ts), sb = __ldg(b_ts);  // factor: a power of two
+  const float sa = factor * a_ts[0], sb = b_ts[0];  // factor: a power of two
   const int q_n = (N + 3) / 4;
   const long long n = (long long)M * q_n;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -478,7 +476,7 @@ sum_parts_kernel(const float* __restrict__ parts, int splits, long long part_str
     float s[4] = {0.0f, 0.0f, 0.0f, 0.0f}, e[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 8
     for (int j = 0; j < splits; ++j) {
-      const float4 v4 = __ldg(reinterpret_cast<const float4*>(p + j * part_stride));
+      const float4 v4 = *reinterpret_cast<const float4*>(p + j * part_stride);
       const float v[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
       for (int k = 0; k < 4; ++k) two_sum_add(s[k], e[k], v[k]);

@@ -82,9 +82,8 @@ __device__ __forceinline__ void split_e1m2_word(uint32_t w, uint32_t tmask, uint
 // Threads [0, n_code) split 32 elements (two blocks, 16 code bytes) each;
 // threads [n_code, n_code + n_sf) write one 16-byte line of the scale tiles
 // (tile (rt, kt), lane line l: rows 32j + l for j = 0..3, blocks 4kt..4kt+3).
-__global__ void __launch_bounds__(256) split_native_kernel(const uint8_t* __restrict__ codes,
-                                                           const uint8_t* __restrict__ scales, int64_t rows,
-                                                           int64_t K, uint8_t* __restrict__ main_codes,
+__global__ void __launch_bounds__(256) split_native_kernel(const uint8_t* codes, const uint8_t* scales,
+                                                           int64_t rows, int64_t K, uint8_t* __restrict__ main_codes,
                                                            uint8_t* __restrict__ res_codes, uint8_t* __restrict__ sf,
                                                            int64_t n_code, int64_t n_sf) {
   griddep_wait();
@@ -179,8 +178,8 @@ template <bool kARes, bool kBRes>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 nvf4_gemm_kernel(const __grid_constant__ CUtensorMap tm_am, const __grid_constant__ CUtensorMap tm_ar,
                  const __grid_constant__ CUtensorMap tm_bm, const __grid_constant__ CUtensorMap tm_br,
-                 const uint8_t* __restrict__ a_sf, const uint8_t* __restrict__ b_sf, const float* __restrict__ a_ts,
-                 const float* __restrict__ b_ts, int M, int N, int K, float* __restrict__ C, long long ldc,
+                 const uint8_t* a_sf, const uint8_t* b_sf, const float* a_ts, const float* b_ts, int M, int N,
+                 int K, float* __restrict__ C, long long ldc,
                  int dp_tiles, int chunk_kc, int after_zero, uint32_t* status_word) {
   using L = Layout<kARes, kBRes>;
   constexpr int S = L::kStages;
@@ -353,7 +352,7 @@ nvf4_gemm_kernel(const __grid_constant__ CUtensorMap tm_am, const __grid_constan
     const int q = warp & 3;
     const int cg = (warp - kFirstEpi) >> 2;  // 64-column group
     griddep_wait();
-    const float sa = __ldg(a_ts), sb = __ldg(b_ts);
+    const float sa = a_ts[0], sb = b_ts[0];
     const bool vec_ok = ((ldc & 3) == 0) && ((reinterpret_cast<uintptr_t>(C) & 15) == 0);
     const uint32_t acc_empty_leader = mapa_shared(smem_u32(&bars->acc_empty), 0);
     const uint32_t tbase = tmem_base + (uint32_t)(cg * kEpiCols) + ((uint32_t)(q * 32) << 16);
@@ -564,7 +563,7 @@ __device__ __forceinline__ uint32_t sf_offset(int r) { return (uint32_t)((r & 31
 __global__ void __launch_bounds__(kThreads, 1)
 nvf4_fewrows_kernel(const __grid_constant__ CUtensorMap tm_wc, const __grid_constant__ CUtensorMap tm_ws,
                     const __grid_constant__ CUtensorMap tm_xc, const __grid_constant__ CUtensorMap tm_xs,
-                    const float* __restrict__ a_ts, const float* __restrict__ b_ts, int Mx, int nx, int N, int K,
+                    const float* a_ts, const float* b_ts, int Mx, int nx, int N, int K,
                     float* __restrict__ C, long long ldc, int chunk_units, uint32_t* status_word) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -786,7 +785,7 @@ nvf4_fewrows_kernel(const __grid_constant__ CUtensorMap tm_wc, const __grid_cons
     const int d = q * 32 + lane;
     const int m = d % XR;
     griddep_wait();
-    const float sa = __ldg(a_ts), sb = __ldg(b_ts);
+    const float sa = a_ts[0], sb = b_ts[0];
     const bool vec_ok = ((ldc & 3) == 0) && ((reinterpret_cast<uintptr_t>(C) & 15) == 0);
     const bool mine = q * 32 < 2 * XR && (q * 32) % XR < Mx;
     const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16);

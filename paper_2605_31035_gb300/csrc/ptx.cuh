@@ -49,7 +49,10 @@ __device__ __forceinline__ void griddep_launch_dependents() {
 }
 // Wait until the preceding kernel on the stream has completed and its memory
 // operations are visible (returns at once when this kernel was not launched
-// as a programmatic dependent).
+// as a programmatic dependent).  What that kernel writes is read by ordinary
+// loads: a non-coherent one (ld.global.nc, i.e. __ldg or a const __restrict__
+// parameter) asks that the data be constant from the start of this kernel, and
+// the compiler may move it above the wait.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ float max3f(float a, float b, float c) {
@@ -100,7 +103,7 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
 // ---- wide global memory access ------------------------------------------------
 // 32-byte streaming load (read once, do not keep in L1).
 __device__ __forceinline__ void ldg256_stream(const void* p, uint32_t v[8]) {
-  asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+  asm volatile("ld.global.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]),
                  "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
                : "l"(p));

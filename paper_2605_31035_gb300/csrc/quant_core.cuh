@@ -467,11 +467,11 @@ constexpr uint32_t kRhtScaleBits = 0x3DB504F3u;  // RN(1/sqrt(128))
 
 // Sign masks of this thread's 16 chunk positions 16 * (lane & 7) + e, as bf16
 // word masks (bit 15: element 2j, bit 31: element 2j + 1).
-__device__ __forceinline__ void rht_sign_words(const uint8_t* __restrict__ signs, int lane, uint32_t sw[8]) {
+__device__ __forceinline__ void rht_sign_words(const uint8_t* signs, int lane, uint32_t sw[8]) {
   uint32_t bits = 0;
   if (signs) {
     const int pos = lane & 7;
-    bits = (uint32_t)__ldg(signs + 2 * pos) | ((uint32_t)__ldg(signs + 2 * pos + 1) << 8);
+    bits = (uint32_t)signs[2 * pos] | ((uint32_t)signs[2 * pos + 1] << 8);
   }
 #pragma unroll
   for (int j = 0; j < 8; ++j) sw[j] = (((bits >> (2 * j)) & 1u) << 15) | (((bits >> (2 * j + 1)) & 1u) << 31);

@@ -73,7 +73,7 @@ __device__ __forceinline__ void store_block(uint8_t* __restrict__ codes, uint8_t
 // kernel is bound by instruction issue, and 64-bit index arithmetic was one
 // instruction in thirty).
 template <int kMode, bool kContig, bool kF16, bool kScaled, bool kMarkstein, typename Index>
-__device__ __forceinline__ void quantize_pairs(const uint16_t* __restrict__ x, Index b, Index nthr,
+__device__ __forceinline__ void quantize_pairs(const uint16_t* x, Index b, Index nthr,
                                                Index nblocks, int64_t kblocks, int64_t ldx,
                                                uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
                                                const TensorConsts& tc, const float4* __restrict__ tab,
@@ -95,7 +95,7 @@ __device__ __forceinline__ void quantize_pairs(const uint16_t* __restrict__ x, I
 // The first loads are issued before any set-up work.
 template <int kMode, bool kContig, bool kF16>
 __global__ void __launch_bounds__(kQuantThreads, 4)
-quantize_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, int64_t ldx,
+quantize_kernel(const uint16_t* x, int64_t nblocks, int64_t kblocks, int64_t ldx,
                 uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, float* tensor_scale,
                 const uint32_t* amax_word, int amax_parts, int scale_given, int after_amax) {
   __shared__ float4 tab[128];  // E4M3 code -> {s8, zh, zl, 0} (zh, zl: see div_kd2)
@@ -117,7 +117,7 @@ quantize_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks
     // The amax pass's maxima, one per CTA of it.
     __shared__ uint32_t red[kQuantThreads / 32];
     uint32_t m = 0u;
-    for (int i = threadIdx.x; i < amax_parts; i += kQuantThreads) m = max(m, __ldcg(amax_word + i));
+    for (int i = threadIdx.x; i < amax_parts; i += kQuantThreads) m = max(m, amax_word[i]);
     m = __reduce_max_sync(0xffffffffu, m);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
     __syncthreads();
@@ -152,7 +152,7 @@ constexpr int kSmallCtas = 8, kSmallThreads = 512, kSmallPer = 4;
 
 template <int kMode, bool kContig, int kOut>
 __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads, 1)
-quantize_small_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, int64_t ldx,
+quantize_small_kernel(const uint16_t* x, int64_t nblocks, int64_t kblocks, int64_t ldx,
                       uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, float* tensor_scale, int xr) {
   __shared__ float4 tab[128];
   __shared__ uint32_t red[kSmallThreads / 32], maxes[kSmallCtas], amax;
@@ -220,7 +220,7 @@ quantize_small_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t k
 }
 
 template <int kMode, bool kContig, typename Index>
-__device__ __forceinline__ void rht_pairs(const uint16_t* __restrict__ x, Index b, Index nthr, Index nblocks,
+__device__ __forceinline__ void rht_pairs(const uint16_t* x, Index b, Index nthr, Index nblocks,
                                           int64_t kblocks, int64_t ldx, uint8_t* __restrict__ codes,
                                           uint8_t* __restrict__ scales, const TensorConsts& tc,
                                           const float4* __restrict__ tab, const uint32_t (&sw)[8], int lane,
@@ -253,8 +253,8 @@ __device__ __forceinline__ void rht_pairs(const uint16_t* __restrict__ x, Index 
 // quantize_kernel); the rotated pairs take 2 CTAs per SM of registers.
 template <int kMode, bool kContig>
 __global__ void __launch_bounds__(kQuantThreads, 2)
-rht_quantize_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, int64_t ldx,
-                    const uint8_t* __restrict__ signs, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
+rht_quantize_kernel(const uint16_t* x, int64_t nblocks, int64_t kblocks, int64_t ldx,
+                    const uint8_t* signs, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
                     float* tensor_scale, const uint32_t* amax_word, int scale_given, int after_amax) {
   __shared__ float4 tab[128];
   if (!after_amax) griddep_wait();
@@ -288,8 +288,8 @@ rht_quantize_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kbl
 // max |y| of the rotated tensor as the bit pattern of a non-negative fp32.
 template <bool kContig>
 __global__ void __launch_bounds__(256)
-rht_amax_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, int64_t ldx,
-                const uint8_t* __restrict__ signs, uint32_t* amax_word) {
+rht_amax_kernel(const uint16_t* x, int64_t nblocks, int64_t kblocks, int64_t ldx,
+                const uint8_t* signs, uint32_t* amax_word) {
   griddep_launch_dependents();
   const int lane = threadIdx.x & 31;
   uint32_t sw[8];
@@ -369,7 +369,7 @@ __device__ __forceinline__ const uint16_t* amax_src(const uint16_t* x, int64_t b
 // are about 2.5 us of a call).
 template <bool kContig, bool kParts>
 __global__ void __launch_bounds__(256, kAmaxCtas)
-amax_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, int64_t ldx,
+amax_kernel(const uint16_t* x, int64_t nblocks, int64_t kblocks, int64_t ldx,
             uint32_t* amax_word) {
   if (kParts) griddep_wait();
   uint32_t m = 0;

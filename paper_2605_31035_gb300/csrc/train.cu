@@ -42,7 +42,7 @@ constexpr int kColRows = 64;            // rows per tile (four 16-row blocks)
 
 template <int kMode, bool kSR>
 __global__ void __launch_bounds__(kColThreads, kSR ? 3 : 4)
-quantize_colwise_kernel(const uint16_t* __restrict__ x, int64_t R, int64_t C, int64_t ldx,
+quantize_colwise_kernel(const uint16_t* x, int64_t R, int64_t C, int64_t ldx,
                         uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, float* tensor_scale,
                         const uint32_t* amax_word, int scale_given, uint64_t seed, uint64_t offset) {
   __shared__ float4 tab[128];
@@ -72,8 +72,8 @@ quantize_colwise_kernel(const uint16_t* __restrict__ x, int64_t R, int64_t C, in
       const int pr = q / (kColThreads / 8), ch = q % (kColThreads / 8);
       uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
       if (r0 + 2 * pr < R && c0 + ch * 8 < C) {
-        a = __ldg(reinterpret_cast<const uint4*>(x + (r0 + 2 * pr) * ldx + c0 + ch * 8));
-        b = __ldg(reinterpret_cast<const uint4*>(x + (r0 + 2 * pr + 1) * ldx + c0 + ch * 8));
+        a = *reinterpret_cast<const uint4*>(x + (r0 + 2 * pr) * ldx + c0 + ch * 8);
+        b = *reinterpret_cast<const uint4*>(x + (r0 + 2 * pr + 1) * ldx + c0 + ch * 8);
       }
       uint4* dst = reinterpret_cast<uint4*>(&pairs[pr][ch * 8]);
       dst[0] = make_uint4(prmt(a.x, b.x, 0x5410u), prmt(a.x, b.x, 0x7632u), prmt(a.y, b.y, 0x5410u),
@@ -132,7 +132,7 @@ quantize_colwise_kernel(const uint16_t* __restrict__ x, int64_t R, int64_t C, in
 // Grid-stride loop of the stochastic-rounding quantizer with the division
 // method fixed; the next block's load is in flight while a block is quantized.
 template <int kMode, bool kContig, bool kScaled, bool kMarkstein>
-__device__ __forceinline__ void sr_loop(const uint16_t* __restrict__ x, int64_t b, int64_t nthr, int64_t nblocks,
+__device__ __forceinline__ void sr_loop(const uint16_t* x, int64_t b, int64_t nthr, int64_t nblocks,
                                         int64_t kblocks, int64_t ldx, uint8_t* __restrict__ codes,
                                         uint8_t* __restrict__ scales, const TensorConsts& tc,
                                         const float4* __restrict__ tab, uint64_t seed, uint64_t offset) {
@@ -155,7 +155,7 @@ __device__ __forceinline__ void sr_loop(const uint16_t* __restrict__ x, int64_t 
 // is 16 b (row-major over [rows][K]).
 template <int kMode, bool kContig>
 __global__ void __launch_bounds__(256, 3)
-quantize_sr_kernel(const uint16_t* __restrict__ x, int64_t nblocks, int64_t kblocks, int64_t ldx,
+quantize_sr_kernel(const uint16_t* x, int64_t nblocks, int64_t kblocks, int64_t ldx,
                    uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, float* tensor_scale,
                    const uint32_t* amax_word, int scale_given, uint64_t seed, uint64_t offset) {
   __shared__ float4 tab[128];
@@ -175,7 +175,7 @@ constexpr int k2dThreads = 256;
 
 template <int kMode>
 __global__ void __launch_bounds__(k2dThreads, 4)
-quantize_2d_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t K, int64_t ldx,
+quantize_2d_kernel(const uint16_t* x, int64_t rows, int64_t K, int64_t ldx,
                    uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, float* tensor_scale,
                    const uint32_t* amax_word, int scale_given) {
   __shared__ float4 tab[128];
@@ -250,8 +250,8 @@ __device__ __forceinline__ void butterfly(u64 (&v)[n]) {
 
 template <int kMode, bool kAmax>
 __global__ void __launch_bounds__(32 * kCrWarps, 4)
-quantize_colwise_rht_kernel(const uint16_t* __restrict__ x, int64_t R, int64_t C, int64_t ldx,
-                            const uint8_t* __restrict__ signs, uint8_t* __restrict__ codes,
+quantize_colwise_rht_kernel(const uint16_t* x, int64_t R, int64_t C, int64_t ldx,
+                            const uint8_t* signs, uint8_t* __restrict__ codes,
                             uint8_t* __restrict__ scales, float* tensor_scale, uint32_t* amax_word, int scale_given) {
   __shared__ float4 tab[128];
   __shared__ __align__(16) float tiles_s[kCrWarps][kCrTile];
@@ -267,7 +267,7 @@ quantize_colwise_rht_kernel(const uint16_t* __restrict__ x, int64_t R, int64_t C
   if (signs)
 #pragma unroll
     for (int h = 0; h < 2; ++h)
-      bits[h] = (uint32_t)__ldg(signs + 2 * (g + 4 * h)) | ((uint32_t)__ldg(signs + 2 * (g + 4 * h) + 1) << 8);
+      bits[h] = (uint32_t)signs[2 * (g + 4 * h)] | ((uint32_t)signs[2 * (g + 4 * h) + 1] << 8);
   TensorConsts tc{};
   if (!kAmax) {
     tc = tensor_consts(tensor_scale, amax_word, scale_given);
@@ -286,7 +286,7 @@ quantize_colwise_rht_kernel(const uint16_t* __restrict__ x, int64_t R, int64_t C
     for (int h = 0; h < 2; ++h)
 #pragma unroll
       for (int i = 0; i < 16; ++i)
-        w[h][i] = __ldg(reinterpret_cast<const uint32_t*>(src + (16 * (g + 4 * h) + i) * ldx));
+        w[h][i] = *reinterpret_cast<const uint32_t*>(src + (16 * (g + 4 * h) + i) * ldx);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {  // strides 1 to 8 of blocks g and g + 4
       u64 v[16];

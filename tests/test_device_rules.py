@@ -46,3 +46,23 @@ def test_cluster_barrier_before_remote_shared_memory(name, body):
     barrier = re.search(r"\bcluster_(sync|wait)\s*\(\s*\)", body)
     remote = re.search(r"\bst_cluster_\w+\s*\(|\bmbar_arrive_cluster\s*\(|\bmma_commit_pair\s*\(", body)
     assert barrier and remote and barrier.start() < remote.start(), name
+
+
+# A programmatic dependent runs while the kernel before it still writes, so
+# nothing it reads may go through the non-coherent path, whose data must be
+# constant for the whole kernel and whose loads may be moved above the wait.
+DEPENDENT = [k for k in KERNELS if "griddep_wait" in k[3]]
+
+
+@pytest.mark.parametrize("params,body", [k[2:] for k in DEPENDENT], ids=[k[1] for k in DEPENDENT])
+def test_dependents_read_coherently(params, body):
+    assert not re.search(r"__ld(g|cg|ca|cs|lu)\s*\(", body)
+    assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", params)
+
+
+def test_shared_device_code_reads_coherently():
+    for f in sorted(os.listdir(CSRC)):
+        text = strip_comments(open(os.path.join(CSRC, f)).read())
+        assert "ld.global.nc" not in text, f
+        if f.endswith(".cuh"):
+            assert "__ldg" not in text, f
