@@ -6,6 +6,7 @@ All arithmetic runs in the library's CUDA kernels; there is no fallback.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 from dataclasses import dataclass
@@ -206,35 +207,78 @@ class QTensor:
         return self.codes.shape[1] * 2
 
 
-def _scratch(nbytes: int, device):
+# What a call allocates is allocated on the stream it runs on.  The allocator
+# hands a freed block out again in the order of the stream it belongs to: a block
+# of the current stream may still be read or written by that stream's pending
+# kernels, which nothing orders before a call on another stream.
+
+
+def _elsewhere(stream, device) -> bool:
+    """Whether a call's stream is another than the current one."""
+    return stream is not None and stream.cuda_stream != torch.cuda.current_stream(device).cuda_stream
+
+
+def _on(stream, device):
+    """The context of a call's allocations and copies."""
+    if not _elsewhere(stream, device):
+        return contextlib.nullcontext()
+    return torch.cuda.stream(_torch_stream(stream, device))
+
+
+def _torch_stream(stream, device):
+    """A stream argument may be any object with a `cuda_stream`."""
+    return stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream, device)
+
+
+def _empty(shape, dtype, device, stream, scratch: bool = False):
+    """Uninitialised memory of a call on `stream`: a result, the caller's to use
+    and to drop on the current stream, or scratch."""
+    if not _elsewhere(stream, device):
+        return torch.empty(shape, dtype=dtype, device=device)
+    with _on(stream, device):
+        t = torch.empty(shape, dtype=dtype, device=device)
+    if not scratch:
+        t.record_stream(torch.cuda.current_stream(device))
+    return t
+
+
+def _scratch(nbytes: int, device, stream):
     """Scratch memory that a call takes and returns, or None where the device
     has no room for it (the caller then goes without)."""
     try:
-        return torch.empty(nbytes, dtype=torch.uint8, device=device)
+        return _empty(nbytes, torch.uint8, device, stream, scratch=True)
     except torch.OutOfMemoryError:
         return None
 
 
-def empty_qtensor(rows: int, K: int, device) -> QTensor:
-    return QTensor(torch.empty(rows, K // 2, dtype=torch.uint8, device=device),
-                   torch.empty(rows, K // 16, dtype=torch.uint8, device=device),
-                   torch.empty(1, dtype=torch.float32, device=device))
+def _set_scale(dst, tensor_scale, device, stream):
+    """Copy a given tensor scale, on the call's stream, before its kernels."""
+    with _on(stream, device):
+        dst.copy_(tensor_scale.reshape(1))
+    if _elsewhere(stream, device) and tensor_scale.is_cuda:
+        tensor_scale.record_stream(_torch_stream(stream, device))  # the caller may drop it at once
 
 
-def _quantizer_args(x, rows: int, K: int, tensor_scale, out, workspace):
+def empty_qtensor(rows: int, K: int, device, stream=None) -> QTensor:
+    return QTensor(_empty((rows, K // 2), torch.uint8, device, stream),
+                   _empty((rows, K // 16), torch.uint8, device, stream),
+                   _empty(1, torch.float32, device, stream))
+
+
+def _quantizer_args(x, rows: int, K: int, tensor_scale, out, workspace, stream):
     """Outputs and scratch of a quantizer call whose result is [rows, K]:
     (QTensor, workspace or None, scale flag)."""
     if out is None:
-        q = empty_qtensor(rows, K, x.device)
+        q = empty_qtensor(rows, K, x.device, stream)
     else:
         q = out
         _check_qtensor(q, rows, K, x.device, "out")
     if tensor_scale is not None:
         _check_given_scale(tensor_scale)
-        q.tensor_scale.copy_(tensor_scale.reshape(1))
+        _set_scale(q.tensor_scale, tensor_scale, x.device, stream)
         return q, None, SCALE_GIVEN
     if workspace is None:
-        return q, torch.empty(1, dtype=torch.int32, device=x.device), SCALE_COMPUTE
+        return q, _empty(1, torch.int32, x.device, stream, scratch=True), SCALE_COMPUTE
     _check_workspace(workspace, x.device)
     return q, workspace, SCALE_COMPUTE
 
@@ -249,7 +293,7 @@ def mixfp4_quantize(x: torch.Tensor, mode: int = MODE_MIX, tensor_scale: torch.T
     """
     _check_x(x)
     rows, K = x.shape
-    q, ws, flag = _quantizer_args(x, rows, K, tensor_scale, out, workspace)
+    q, ws, flag = _quantizer_args(x, rows, K, tensor_scale, out, workspace, stream)
     st = lib().mixfp4_quantize(_ptr(x), DTYPE_BF16, rows, K, x.stride(0), _ptr(q.codes), _ptr(q.scales),
                                _ptr(q.tensor_scale), _ptr(ws), int(mode), flag, _stream(stream))
     _check("mixfp4_quantize", st)
@@ -265,7 +309,7 @@ def mixfp4_quantize_rht(x: torch.Tensor, signs: torch.Tensor | None = None, mode
     _check_x(x)
     _check_signs(signs)
     rows, K = x.shape
-    q, ws, flag = _quantizer_args(x, rows, K, tensor_scale, out, workspace)
+    q, ws, flag = _quantizer_args(x, rows, K, tensor_scale, out, workspace, stream)
     st = lib().mixfp4_quantize_rht(_ptr(x), DTYPE_BF16, rows, K, x.stride(0), _ptr(signs), _ptr(q.codes),
                                    _ptr(q.scales), _ptr(q.tensor_scale), _ptr(ws), int(mode), flag,
                                    _stream(stream))
@@ -281,7 +325,7 @@ def mixfp4_quantize_colwise(x: torch.Tensor, mode: int = MODE_MIX, tensor_scale:
     X^T, codes [C, R/2], scales [C, R/16]."""
     _check_x(x)
     R, C = x.shape
-    q, ws, flag = _quantizer_args(x, C, R, tensor_scale, out, workspace)
+    q, ws, flag = _quantizer_args(x, C, R, tensor_scale, out, workspace, stream)
     st = lib().mixfp4_quantize_colwise(_ptr(x), DTYPE_BF16, R, C, x.stride(0), _ptr(q.codes), _ptr(q.scales),
                                        _ptr(q.tensor_scale), _ptr(ws), int(mode), flag, _stream(stream))
     _check("mixfp4_quantize_colwise", st)
@@ -296,7 +340,7 @@ def mixfp4_quantize_colwise_rht(x: torch.Tensor, signs: torch.Tensor | None = No
     _check_x(x)
     _check_signs(signs)
     R, C = x.shape
-    q, ws, flag = _quantizer_args(x, C, R, tensor_scale, out, workspace)
+    q, ws, flag = _quantizer_args(x, C, R, tensor_scale, out, workspace, stream)
     st = lib().mixfp4_quantize_colwise_rht(_ptr(x), DTYPE_BF16, R, C, x.stride(0), _ptr(signs), _ptr(q.codes),
                                            _ptr(q.scales), _ptr(q.tensor_scale), _ptr(ws), int(mode), flag,
                                            _stream(stream))
@@ -311,7 +355,7 @@ def mixfp4_quantize_sr(x: torch.Tensor, seed: int, offset: int = 0, mode: int = 
     stochastic rounding of the codes drawn from (seed, offset)."""
     _check_x(x)
     rows, K = x.shape
-    q, ws, flag = _quantizer_args(x, K if colwise else rows, rows if colwise else K, tensor_scale, out, workspace)
+    q, ws, flag = _quantizer_args(x, K if colwise else rows, rows if colwise else K, tensor_scale, out, workspace, stream)
     fn = lib().mixfp4_quantize_colwise_sr if colwise else lib().mixfp4_quantize_sr
     st = fn(_ptr(x), DTYPE_BF16, rows, K, x.stride(0), _ptr(q.codes), _ptr(q.scales), _ptr(q.tensor_scale),
             _ptr(ws), int(mode), flag, int(seed) & (2 ** 64 - 1), int(offset) & (2 ** 64 - 1), _stream(stream))
@@ -326,7 +370,7 @@ def mixfp4_quantize_2d(x: torch.Tensor, mode: int = MODE_MIX, tensor_scale: torc
     and format per tile, repeated on the tile's rows)."""
     _check_x(x)
     rows, K = x.shape
-    q, ws, flag = _quantizer_args(x, rows, K, tensor_scale, out, workspace)
+    q, ws, flag = _quantizer_args(x, rows, K, tensor_scale, out, workspace, stream)
     st = lib().mixfp4_quantize_2d(_ptr(x), DTYPE_BF16, rows, K, x.stride(0), _ptr(q.codes), _ptr(q.scales),
                                   _ptr(q.tensor_scale), _ptr(ws), int(mode), flag, _stream(stream))
     _check("mixfp4_quantize_2d", st)
@@ -338,8 +382,8 @@ def mixfp4_transpose_2d(q: QTensor, out: QTensor | None = None, stream=None) -> 
     the tensor scale is shared with the input."""
     _check_operand(q, "q")
     if out is None:
-        t = QTensor(torch.empty(q.K, q.rows // 2, dtype=torch.uint8, device=q.codes.device),
-                    torch.empty(q.K, q.rows // 16, dtype=torch.uint8, device=q.codes.device), q.tensor_scale)
+        t = QTensor(_empty((q.K, q.rows // 2), torch.uint8, q.codes.device, stream),
+                    _empty((q.K, q.rows // 16), torch.uint8, q.codes.device, stream), q.tensor_scale)
     else:
         t = out
         _check_u8(t.codes, (q.K, q.rows // 2), q.codes.device, "out.codes")
@@ -362,25 +406,24 @@ def mixfp4_fake_quantize(x: torch.Tensor, candidates: int, block: int = 16, out_
     _require(out_dtype in (torch.float32, torch.bfloat16), "out_dtype must be torch.float32 or torch.bfloat16")
     _require(block in (8, 16, 32, 64), "block must be 8, 16, 32 or 64")
     rows, K = x.shape
-    o = out if out is not None else torch.empty(rows, K, dtype=out_dtype, device=x.device)
+    o = out if out is not None else _empty((rows, K), out_dtype, x.device, stream)
     _check_dev(o, x.device, "out")
     _require(o.dtype == out_dtype and o.dim() == 2 and o.shape == x.shape and o.stride(1) == 1,
              "out must be a [rows, K] tensor of out_dtype with unit column stride")
     ch = None
     if want_choice:
-        ch = choice if choice is not None else torch.empty(rows, K // block, dtype=torch.uint8,
-                                                           device=x.device)
+        ch = choice if choice is not None else _empty((rows, K // block), torch.uint8, x.device, stream)
         _check_dev(ch, x.device, "choice")
         _require(ch.dtype == torch.uint8 and ch.is_contiguous() and ch.numel() == rows * (K // block),
                  "choice must be a dense uint8 [rows, K / block] tensor")
     _check_given_scale(tensor_scale)
-    ts = torch.empty(1, dtype=torch.float32, device=x.device)
+    ts = _empty(1, torch.float32, x.device, stream)
     given = tensor_scale is not None
     if given:
-        ts.copy_(tensor_scale.reshape(1))
+        _set_scale(ts, tensor_scale, x.device, stream)
     ws = None
     if not given:
-        ws = workspace if workspace is not None else torch.empty(1, dtype=torch.int32, device=x.device)
+        ws = workspace if workspace is not None else _empty(1, torch.int32, x.device, stream, scratch=True)
         _check_workspace(ws, x.device)
     st = lib().mixfp4_fake_quantize(_ptr(x), DTYPE_BF16, rows, K, x.stride(0), int(candidates), int(block),
                                     _ptr(ts), _ptr(ws), SCALE_GIVEN if given else SCALE_COMPUTE, _ptr(o),
@@ -392,7 +435,7 @@ def mixfp4_fake_quantize(x: torch.Tensor, candidates: int, block: int = 16, out_
 
 def mixfp4_dequantize(q: QTensor, out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     _check_operand(q, "q")
-    o = out if out is not None else torch.empty(q.rows, q.K, dtype=torch.float32, device=q.codes.device)
+    o = out if out is not None else _empty((q.rows, q.K), torch.float32, q.codes.device, stream)
     _check_dev(o, q.codes.device, "out")
     _require(o.dtype == torch.float32 and tuple(o.shape) == (q.rows, q.K) and o.is_contiguous(),
              "out must be a dense float32 [rows, K] tensor")
@@ -402,11 +445,13 @@ def mixfp4_dequantize(q: QTensor, out: torch.Tensor | None = None, stream=None) 
     return o
 
 
-def _gemm_out(out, M: int, N: int, device):
+def _gemm_out(out, M: int, N: int, device, stream):
     if out is None:
-        return torch.empty(M, N, dtype=torch.float32, device=device)
+        return _empty((M, N), torch.float32, device, stream)
     _check_c(out, M, N, device)
     return out
+
+
 def gemm_workspace_bytes(M: int, N: int, K: int) -> int:
     """Bytes of scratch memory mixfp4_gemm_ws takes for an M x N x K product (0: none)."""
     n = ctypes.c_int64(0)
@@ -421,21 +466,18 @@ def mixfp4_gemm(a: QTensor, b: QTensor, out: torch.Tensor | None = None,
     _check_operand(b, "b")
     _require(a.K == b.K and a.codes.device == b.codes.device, "operands must share K and device")
     M, N, K = a.rows, b.rows, a.K
-    C = _gemm_out(out, M, N, a.codes.device)
+    C = _gemm_out(out, M, N, a.codes.device, stream)
     _check_status(status_word, a.codes.device)
     ws_bytes = gemm_workspace_bytes(M, N, K) if K % 256 == 0 else 0
-    ws = _scratch(ws_bytes, a.codes.device) if ws_bytes > 0 else None
+    ws = _scratch(ws_bytes, a.codes.device, stream) if ws_bytes > 0 else None
     _check("mixfp4_gemm", _gemm_ws(a, b, C, ws, status_word, stream))
     return C
 
 
 def _gemm_ws(a: QTensor, b: QTensor, C, ws, status_word, stream) -> int:
-    st = lib().mixfp4_gemm_ws(_ptr(a.codes), _ptr(a.scales), _ptr(a.tensor_scale), _ptr(b.codes), _ptr(b.scales),
-                              _ptr(b.tensor_scale), a.rows, b.rows, a.K, _ptr(C), C.stride(0), _ptr(ws),
-                              0 if ws is None else ws.numel(), _ptr(status_word), _stream(stream))
-    if ws is not None and stream is not None:
-        ws.record_stream(stream)  # allocated on the current stream, used on the caller's
-    return st
+    return lib().mixfp4_gemm_ws(_ptr(a.codes), _ptr(a.scales), _ptr(a.tensor_scale), _ptr(b.codes), _ptr(b.scales),
+                                _ptr(b.tensor_scale), a.rows, b.rows, a.K, _ptr(C), C.stride(0), _ptr(ws),
+                                0 if ws is None else ws.numel(), _ptr(status_word), _stream(stream))
 
 
 @dataclass
@@ -484,9 +526,9 @@ def mixfp4_split_native(q: QTensor, keep_residual: bool = True, out: NativeTenso
         _check_native(out, q.rows, q.K, dev, "out")
         main, res, sf = out.main, out.res, out.sf
     else:
-        main = torch.empty_like(q.codes)
-        res = torch.empty_like(q.codes)
-        sf = torch.empty(sf_tiled_bytes(q.rows, q.K), dtype=torch.uint8, device=dev)
+        main = _empty(q.codes.shape, torch.uint8, dev, stream)
+        res = _empty(q.codes.shape, torch.uint8, dev, stream)
+        sf = _empty(sf_tiled_bytes(q.rows, q.K), torch.uint8, dev, stream)
     st = lib().mixfp4_split_native(_ptr(q.codes), _ptr(q.scales), q.rows, q.K, _ptr(main), _ptr(res), _ptr(sf),
                                    _stream(stream))
     _check("mixfp4_split_native", st)
@@ -503,7 +545,7 @@ def mixfp4_gemm_native(a: NativeTensor, b: NativeTensor, out: torch.Tensor | Non
     _check_native(b, b.rows, b.K, dev, "b")
     _require(a.K == b.K, "operands must share K")
     M, N, K = a.rows, b.rows, a.K
-    C = _gemm_out(out, M, N, dev)
+    C = _gemm_out(out, M, N, dev, stream)
     _check_status(status_word, dev)
     st = lib().mixfp4_gemm_native(_ptr(a.main), _ptr(a.res), _ptr(a.sf), _ptr(a.tensor_scale),
                                   _ptr(b.main), _ptr(b.res), _ptr(b.sf), _ptr(b.tensor_scale),
@@ -522,10 +564,10 @@ def mixfp4_gemm_native_fewrows(a: QTensor, b: QTensor, out: torch.Tensor | None 
     _require(a.K == b.K and a.rows <= 64 and a.codes.device == b.codes.device,
              "operands must share K and device, and A have at most 64 rows")
     M, N, K = a.rows, b.rows, a.K
-    C = _gemm_out(out, M, N, a.codes.device)
+    C = _gemm_out(out, M, N, a.codes.device, stream)
     _check_status(status_word, a.codes.device)
     ws_bytes = gemm_workspace_bytes(M, N, K) if K % 256 == 0 else 0
-    ws = _scratch(ws_bytes, a.codes.device) if ws_bytes > 0 else None
+    ws = _scratch(ws_bytes, a.codes.device, stream) if ws_bytes > 0 else None
     if ws is not None:
         _check("mixfp4_gemm_native_fewrows", _gemm_ws(a, b, C, ws, status_word, stream))
         return C
@@ -538,7 +580,8 @@ def mixfp4_gemm_native_fewrows(a: QTensor, b: QTensor, out: torch.Tensor | None 
 
 def selftest_bounded_wait(limit_ns: int = 20_000_000, stream=None) -> int:
     """Run the bounded-wait self-test; returns the status bits (0xE when healthy)."""
-    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    with _on(stream, "cuda"):
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
     _check("mixfp4_selftest_bounded_wait",
            lib().mixfp4_selftest_bounded_wait(_ptr(status), int(limit_ns), _stream(stream)))
     torch.cuda.synchronize()
@@ -554,7 +597,8 @@ def selftest_gemm_missed_stage(a: QTensor, b: QTensor, out: torch.Tensor, limit_
     _check_operand(b, "b")
     _require(a.K == b.K and a.codes.device == b.codes.device, "operands must share K and device")
     _check_c(out, a.rows, b.rows, a.codes.device)
-    status = torch.zeros(1, dtype=torch.int32, device=a.codes.device)
+    with _on(stream, a.codes.device):
+        status = torch.zeros(1, dtype=torch.int32, device=a.codes.device)
     _check("mixfp4_selftest_gemm_missed_stage",
            lib().mixfp4_selftest_gemm_missed_stage(_ptr(a.codes), _ptr(a.scales), _ptr(a.tensor_scale),
                                                    _ptr(b.codes), _ptr(b.scales), _ptr(b.tensor_scale), a.rows,
@@ -573,17 +617,15 @@ def linear(x: torch.Tensor, w_q: QTensor, mode: int = MODE_MIX, stream=None) -> 
             and w_q.codes.dim() == 2 and w_q.codes.shape[1] * 2 == K and w_q.codes.device == x.device:
         _check_operand(w_q, "b")
         N = w_q.codes.shape[0]
-        C = torch.empty(M, N, dtype=torch.float32, device=x.device)
+        C = _empty((M, N), torch.float32, x.device, stream)
         # One scratch buffer for the quantized activations (and the parts of a split K).
         n = ctypes.c_int64(0)
         L = lib()
-        ws = _scratch(n.value, x.device) if L.mixfp4_linear_workspace(M, N, K, ctypes.byref(n)) == 0 else None
+        ws = _scratch(n.value, x.device, stream) if L.mixfp4_linear_workspace(M, N, K, ctypes.byref(n)) == 0 else None
         if ws is not None:
             st = L.mixfp4_linear(_ptr(x), DTYPE_BF16, M, K, x.stride(0), int(mode), _ptr(w_q.codes),
                                  _ptr(w_q.scales), _ptr(w_q.tensor_scale), N, _ptr(C), N, _ptr(ws), ws.numel(),
                                  None, _stream(stream))
-            if stream is not None:
-                ws.record_stream(stream)  # allocated on the current stream, used on the caller's
             if st in (0, _ERR_CUDA):
                 _check("mixfp4_linear", st)
                 return C
