@@ -164,6 +164,11 @@ def _check_workspace(ws, device):
                  "workspace must be a dense CUDA tensor of at least 4 bytes")
 
 
+def _check_scratch(ws, device):
+    _check_dev(ws, device, "workspace")
+    _require(ws.is_contiguous(), "workspace must be a dense CUDA tensor")
+
+
 def _check_status(sw, device):
     if sw is not None:
         _check_dev(sw, device, "status_word")
@@ -459,17 +464,43 @@ def gemm_workspace_bytes(M: int, N: int, K: int) -> int:
     return n.value
 
 
+def linear_workspace_bytes(M: int, N: int, K: int) -> int:
+    """Bytes of scratch memory linear() makes use of."""
+    n = ctypes.c_int64(0)
+    _check("mixfp4_linear", lib().mixfp4_linear_workspace(M, N, K, ctypes.byref(n)))
+    return n.value
+
+
+def _bytes(t) -> int:
+    return 0 if t is None else t.numel() * t.element_size()
+
+
+def _gemm_scratch(M: int, N: int, K: int, device, stream, workspace):
+    """The caller's workspace where one is given and large enough, else None
+    (the call then goes without); memory of the call's own otherwise."""
+    n = gemm_workspace_bytes(M, N, K) if K % 256 == 0 else 0
+    if workspace is not None:
+        _check_scratch(workspace, device)
+        return workspace if 0 < n <= _bytes(workspace) else None
+    return _scratch(n, device, stream) if n > 0 else None
+
+
 def mixfp4_gemm(a: QTensor, b: QTensor, out: torch.Tensor | None = None,
-                status_word: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-    """C = A_deq . B_deq^T in fp32; a is M x K, b is N x K."""
+                status_word: torch.Tensor | None = None, stream=None,
+                workspace: torch.Tensor | None = None) -> torch.Tensor:
+    """C = A_deq . B_deq^T in fp32; a is M x K, b is N x K.
+
+    workspace: scratch memory of the caller's, any dense CUDA tensor aligned to
+    256 bytes, free for reuse once the call's work is done.  The call allocates
+    none then: with gemm_workspace_bytes(M, N, K) of it the fast forms run, with
+    less (an empty tensor too) the form that needs none."""
     _check_operand(a, "a")
     _check_operand(b, "b")
     _require(a.K == b.K and a.codes.device == b.codes.device, "operands must share K and device")
     M, N, K = a.rows, b.rows, a.K
     C = _gemm_out(out, M, N, a.codes.device, stream)
     _check_status(status_word, a.codes.device)
-    ws_bytes = gemm_workspace_bytes(M, N, K) if K % 256 == 0 else 0
-    ws = _scratch(ws_bytes, a.codes.device, stream) if ws_bytes > 0 else None
+    ws = _gemm_scratch(M, N, K, a.codes.device, stream, workspace)
     _check("mixfp4_gemm", _gemm_ws(a, b, C, ws, status_word, stream))
     return C
 
@@ -477,7 +508,7 @@ def mixfp4_gemm(a: QTensor, b: QTensor, out: torch.Tensor | None = None,
 def _gemm_ws(a: QTensor, b: QTensor, C, ws, status_word, stream) -> int:
     return lib().mixfp4_gemm_ws(_ptr(a.codes), _ptr(a.scales), _ptr(a.tensor_scale), _ptr(b.codes), _ptr(b.scales),
                                 _ptr(b.tensor_scale), a.rows, b.rows, a.K, _ptr(C), C.stride(0), _ptr(ws),
-                                0 if ws is None else ws.numel(), _ptr(status_word), _stream(stream))
+                                _bytes(ws), _ptr(status_word), _stream(stream))
 
 
 @dataclass
@@ -555,10 +586,12 @@ def mixfp4_gemm_native(a: NativeTensor, b: NativeTensor, out: torch.Tensor | Non
 
 
 def mixfp4_gemm_native_fewrows(a: QTensor, b: QTensor, out: torch.Tensor | None = None,
-                               status_word: torch.Tensor | None = None, stream=None) -> torch.Tensor:
+                               status_word: torch.Tensor | None = None, stream=None,
+                               workspace: torch.Tensor | None = None) -> torch.Tensor:
     """C = A_deq . B_deq^T for a with at most 64 rows, on the block-scaled FP4
     tensor path: the stored codes are the main E2M1 operands, what their E1M2
-    blocks need beside them and the scale tiles are formed on the fly."""
+    blocks need beside them and the scale tiles are formed on the fly.
+    workspace as mixfp4_gemm's."""
     _check_operand(a, "a")
     _check_operand(b, "b")
     _require(a.K == b.K and a.rows <= 64 and a.codes.device == b.codes.device,
@@ -566,8 +599,7 @@ def mixfp4_gemm_native_fewrows(a: QTensor, b: QTensor, out: torch.Tensor | None 
     M, N, K = a.rows, b.rows, a.K
     C = _gemm_out(out, M, N, a.codes.device, stream)
     _check_status(status_word, a.codes.device)
-    ws_bytes = gemm_workspace_bytes(M, N, K) if K % 256 == 0 else 0
-    ws = _scratch(ws_bytes, a.codes.device, stream) if ws_bytes > 0 else None
+    ws = _gemm_scratch(M, N, K, a.codes.device, stream, workspace)
     if ws is not None:
         _check("mixfp4_gemm_native_fewrows", _gemm_ws(a, b, C, ws, status_word, stream))
         return C
@@ -608,10 +640,17 @@ def selftest_gemm_missed_stage(a: QTensor, b: QTensor, out: torch.Tensor, limit_
     return int(status.item())
 
 
-def linear(x: torch.Tensor, w_q: QTensor, mode: int = MODE_MIX, stream=None) -> torch.Tensor:
+def linear(x: torch.Tensor, w_q: QTensor, mode: int = MODE_MIX, stream=None,
+           workspace: torch.Tensor | None = None) -> torch.Tensor:
     """W4A4 linear: quantize the activations online, then the MixFP4 GEMM with
-    pre-quantized weights.  Returns x_deq . w_deq^T in fp32."""
+    pre-quantized weights.  Returns x_deq . w_deq^T in fp32.
+
+    workspace: scratch memory of the caller's as mixfp4_gemm's, of
+    linear_workspace_bytes(M, N, K); with less the layer runs as its two calls,
+    the GEMM with this workspace."""
     _check_x(x)
+    if workspace is not None:
+        _check_scratch(workspace, x.device)
     M, K = x.shape
     if M > 0 and K > 0 and isinstance(w_q, QTensor) and isinstance(w_q.codes, torch.Tensor) \
             and w_q.codes.dim() == 2 and w_q.codes.shape[1] * 2 == K and w_q.codes.device == x.device:
@@ -621,13 +660,18 @@ def linear(x: torch.Tensor, w_q: QTensor, mode: int = MODE_MIX, stream=None) -> 
         # One scratch buffer for the quantized activations (and the parts of a split K).
         n = ctypes.c_int64(0)
         L = lib()
-        ws = _scratch(n.value, x.device, stream) if L.mixfp4_linear_workspace(M, N, K, ctypes.byref(n)) == 0 else None
+        ws = None
+        if L.mixfp4_linear_workspace(M, N, K, ctypes.byref(n)) == 0:
+            if workspace is None:
+                ws = _scratch(n.value, x.device, stream)
+            elif _bytes(workspace) >= n.value:
+                ws = workspace
         if ws is not None:
             st = L.mixfp4_linear(_ptr(x), DTYPE_BF16, M, K, x.stride(0), int(mode), _ptr(w_q.codes),
-                                 _ptr(w_q.scales), _ptr(w_q.tensor_scale), N, _ptr(C), N, _ptr(ws), ws.numel(),
+                                 _ptr(w_q.scales), _ptr(w_q.tensor_scale), N, _ptr(C), N, _ptr(ws), _bytes(ws),
                                  None, _stream(stream))
             if st in (0, _ERR_CUDA):
                 _check("mixfp4_linear", st)
                 return C
             # Refused, with nothing enqueued: the two calls below say which one refuses it, and why.
-    return mixfp4_gemm(mixfp4_quantize(x, mode, stream=stream), w_q, stream=stream)
+    return mixfp4_gemm(mixfp4_quantize(x, mode, stream=stream), w_q, stream=stream, workspace=workspace)

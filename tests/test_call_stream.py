@@ -102,3 +102,31 @@ def test_current_stream_needs_no_recording(calls, name):
         CALLS[name](ops, stream)
     assert all(e[2] == 1 for e in log if e[0] in ("empty", "copy"))
     assert not [e for e in log if e[0] == "record"]
+
+
+WITH_WORKSPACE = {
+    "gemm": lambda o, w: o.mixfp4_gemm(qt(o, 80, 256), qt(o, 16, 256), out=torch.zeros(80, 16), workspace=w),
+    "fewrows": lambda o, w: o.mixfp4_gemm_native_fewrows(qt(o, 8, 256), qt(o, 16, 256), out=torch.zeros(8, 16),
+                                                         workspace=w),
+}
+
+
+@pytest.mark.parametrize("nbytes", [0, 4095, 4096, 10000])
+@pytest.mark.parametrize("name", WITH_WORKSPACE)
+def test_a_given_workspace_leaves_nothing_to_allocate(calls, name, nbytes):
+    """Output and workspace the caller's: no allocation, whether the workspace is large enough or not."""
+    ops, log = calls
+    WITH_WORKSPACE[name](ops, torch.zeros(nbytes, dtype=torch.uint8))
+    assert not [e for e in log if e[0] == "empty"]
+    # The library gets the workspace, or (native few rows) the form that needs none runs.
+    native_form = name == "fewrows" and nbytes < 4096
+    assert log[-1][0] == ("mixfp4_gemm_native_fewrows" if native_form else "mixfp4_gemm_ws")
+
+
+def test_linear_with_a_workspace_allocates_its_result_only(calls):
+    ops, log = calls
+    x, w = torch.zeros(8, 256, dtype=torch.bfloat16), qt(ops, 16, 256)
+    ops.linear(x, w, workspace=torch.zeros(4096, dtype=torch.uint8))
+    assert [e[1] for e in log if e[0] == "empty"] == [(8, 16)]
+    with pytest.raises(ValueError, match="workspace"):
+        ops.linear(x, w, workspace=torch.zeros(64, 128, dtype=torch.uint8).t())
