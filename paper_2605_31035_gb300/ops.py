@@ -652,6 +652,7 @@ def linear(x: torch.Tensor, w_q: QTensor, mode: int = MODE_MIX, stream=None,
     if workspace is not None:
         _check_scratch(workspace, x.device)
     M, K = x.shape
+    C = None
     if M > 0 and K > 0 and isinstance(w_q, QTensor) and isinstance(w_q.codes, torch.Tensor) \
             and w_q.codes.dim() == 2 and w_q.codes.shape[1] * 2 == K and w_q.codes.device == x.device:
         _check_operand(w_q, "b")
@@ -674,4 +675,4 @@ def linear(x: torch.Tensor, w_q: QTensor, mode: int = MODE_MIX, stream=None,
                 _check("mixfp4_linear", st)
                 return C
             # Refused, with nothing enqueued: the two calls below say which one refuses it, and why.
-    return mixfp4_gemm(mixfp4_quantize(x, mode, stream=stream), w_q, stream=stream, workspace=workspace)
+    return mixfp4_gemm(mixfp4_quantize(x, mode, stream=stream), w_q, out=C, stream=stream, workspace=workspace)

@@ -130,3 +130,13 @@ def test_linear_with_a_workspace_allocates_its_result_only(calls):
     assert [e[1] for e in log if e[0] == "empty"] == [(8, 16)]
     with pytest.raises(ValueError, match="workspace"):
         ops.linear(x, w, workspace=torch.zeros(64, 128, dtype=torch.uint8).t())
+
+
+def test_linear_without_room_for_scratch_makes_its_result_once(calls, monkeypatch):
+    """Where the device has no room left for scratch, a second result would not
+    fit either: the two calls write the one already made."""
+    ops, log = calls
+    monkeypatch.setattr(ops, "_scratch", lambda *args: None)
+    y = ops.linear(torch.zeros(80, 256, dtype=torch.bfloat16), qt(ops, 16, 256))
+    assert [e[1] for e in log if e[0] == "empty"].count((80, 16)) == 1 and y.shape == (80, 16)
+    assert [e[0] for e in log if e[0].startswith("mixfp4")] == ["mixfp4_quantize", "mixfp4_gemm_ws"]
