@@ -137,6 +137,6 @@ def test_linear_without_room_for_scratch_makes_its_result_once(calls, monkeypatc
     fit either: the two calls write the one already made."""
     ops, log = calls
     monkeypatch.setattr(ops, "_scratch", lambda *args: None)
-    y = ops.linear(torch.zeros(80, 256, dtype=torch.bfloat16), qt(ops, 16, 256))
-    assert [e[1] for e in log if e[0] == "empty"].count((80, 16)) == 1 and y.shape == (80, 16)
+    y = ops.linear(torch.zeros(80, 256, dtype=torch.bfloat16), qt(ops, 24, 256))
+    assert [e[1] for e in log if e[0] == "empty"].count((80, 24)) == 1 and y.shape == (80, 24)
     assert [e[0] for e in log if e[0].startswith("mixfp4")] == ["mixfp4_quantize", "mixfp4_gemm_ws"]
