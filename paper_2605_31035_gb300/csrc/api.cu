@@ -302,9 +302,9 @@ constexpr int64_t kLinearHeader = mixfp4::kMaxAmaxParts * 4 + 256;
 constexpr int64_t kLinearExtra = 16384;  // bytes mixfp4_linear needs beyond 2 M K (mixfp4.h)
 static_assert(kLinearHeader <= kLinearExtra, "linear workspace");
 
-// Up to 64 rows: the codes, the block scales, then (at the returned offset)
-// launch_fewrows' own scratch.
-int64_t few_rows_offset(int64_t M, int64_t K) { return (kLinearHeader + M * (K / 2) + M * (K / 16) + 255) / 256 * 256; }
+// As codes: the codes, the block scales, then (at the returned offset) the
+// GEMM's own scratch.
+int64_t codes_end(int64_t M, int64_t K) { return (kLinearHeader + M * (K / 2) + M * (K / 16) + 255) / 256 * 256; }
 
 // Shared body of the decode-path GEMM entry points.
 int gemm_impl(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_ts, const uint8_t* b_codes,
@@ -379,7 +379,7 @@ int mixfp4_linear_workspace(int64_t M, int64_t N, int64_t K, int64_t* bytes) {
   if (M > 64) {
     *bytes += mixfp4::gemm_f16a_parts_bytes(M, N, K);
   } else {
-    const int64_t few = few_rows_offset(M, K) + mixfp4::fewrows_scratch_bytes(M, N, K);
+    const int64_t few = codes_end(M, K) + mixfp4::fewrows_scratch_bytes(M, N, K);
     if (few > *bytes) *bytes = few;
   }
   return MIXFP4_OK;
@@ -411,11 +411,11 @@ int mixfp4_linear(const void* x, int dtype, int64_t M, int64_t K, int64_t ldx, i
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (status_word && cudaMemsetAsync(status_word, 0, sizeof(uint32_t), s) != cudaSuccess) return MIXFP4_ERR_CUDA;
   const uint16_t* xb = static_cast<const uint16_t*>(x);
-  if (M <= 64) {
-    const int64_t off = few_rows_offset(M, K), room = workspace_bytes - off;
+  if (M <= 64 || !mixfp4::linear_predecode_pays(M, N, K)) {
+    const int64_t off = codes_end(M, K), room = workspace_bytes - off;
     uint8_t* scratch = static_cast<uint8_t*>(workspace) + off;
     int st = 0;
-    if (room >= mixfp4::fewrows_scratch_bytes(M, N, K) &&
+    if (M <= 64 && room >= mixfp4::fewrows_scratch_bytes(M, N, K) &&
         mixfp4::launch_linear_fewrows(xb, M, K, ldx, mode, x_ts, w_codes, w_scales, w_ts, N, C, ldc, scratch,
                                       status_word, s, &st))
       return st ? st : launch_status();

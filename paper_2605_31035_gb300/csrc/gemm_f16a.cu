@@ -521,6 +521,20 @@ bool gemm_predecode_pays(int64_t M, int64_t N, int64_t K) {
   return 0.07 * stages > 1.8 + 0.45e-6 * (double)M * (double)K;
 }
 
+// The same for the layer (M > 64): whether the quantizer writes f16 values, 2 bytes
+// an element, for this GEMM, or codes and scales, 0.56 bytes, for gemm.cu's.  Here
+// no pass is saved by the codes, only bytes, so this GEMM is the rule.  With one
+// column of tiles (N <= 256) gemm.cu decodes A only once as well, and this GEMM has
+// nothing over it but its split of K, for up to half a wave of tiles.  f16 / codes,
+// L2 flushed, us: 32768 x 64 x 4096 209 / 190, 32768 x 256 x 8192 409 / 363, 16384 x 256 x
+// 2560 79 / 75; with K split or below 2^25 elements 8192 x 64 x 14336 190 / 203,
+// 20000 x 64 x 1024 46 / 48, 65536 x 64 x 256 42 / 46; with two columns 32768 x 300 x 8192
+// 429 / 437, 16384 x 384 x 4096 130 / 126.
+bool linear_predecode_pays(int64_t M, int64_t N, int64_t K) {
+  const int64_t pairs = num_sms() / 2, tiles = (M + 255) / 256;
+  return N > 256 || 2 * tiles <= pairs || M * K < (1ll << 25);
+}
+
 namespace {
 
 struct Plan {

@@ -58,6 +58,7 @@ int launch_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const float* a_
 int launch_decode_f16(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K, void* out,
                       cudaStream_t stream);
 bool gemm_predecode_pays(int64_t M, int64_t N, int64_t K);
+bool linear_predecode_pays(int64_t M, int64_t N, int64_t K);
 int launch_gemm_f16a(const void* a_f16, const float* a_ts, const uint8_t* b_codes, const uint8_t* b_scales,
                      const float* b_ts, int64_t M, int64_t N, int64_t K, float* C, int64_t ldc, void* parts,
                      int64_t parts_room, uint32_t* status_word, cudaStream_t stream);

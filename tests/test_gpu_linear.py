@@ -43,3 +43,27 @@ def test_linear_empty_and_refusals():
         ops.linear(torch.zeros(4, 272, dtype=torch.bfloat16, device=DEV), ops.empty_qtensor(8, 272, DEV))
     with pytest.raises(ops.MixFP4Error, match="misaligned"):         # x not 32-byte aligned
         ops.linear(torch.zeros(4, 272, dtype=torch.bfloat16, device=DEV)[:, 8:264], w)
+
+
+# Many rows and one column of weight tiles (N <= 256): the activations stay codes,
+# which the GEMM decodes once, instead of 2 bytes an element.  Both sides of each
+# bound: half a wave of 256-row tiles (one tile more than half of the pairs), 2^25
+# elements, 256 columns; ragged rows, a row stride above K, every mode.
+@pytest.mark.parametrize("tiles,extra,N,K,mode,pad,codes", [
+    (0, 1, 256, 4096, 0, 0, True), (0, 0, 256, 4096, 0, 0, False), (0, 1, 257, 4096, 0, 0, False),
+    (10, -3, 1, 2816, 1, 16, True), (0, 1, 64, 3328, 2, 0, False), (0, 7, 100, 4352, 3, 64, True)])
+def test_linear_one_column_of_tiles(tiles, extra, N, K, mode, pad, codes):
+    from paper_2605_31035_gb300 import ops, synth
+    pairs = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    M = (pairs // 2 + tiles) * 256 + extra
+    assert codes == (N <= 256 and 2 * ((M + 255) // 256) > pairs and M * K >= 1 << 25)
+    x = torch.zeros(M, K + pad, dtype=torch.bfloat16, device=DEV)[:, :K]
+    x.copy_(synth.activations(M, K, 8610, 8611))
+    w = ops.mixfp4_quantize(synth.weights(N, K, 8612, 0.02, 0.5).to(DEV), mode)
+    q = ops.mixfp4_quantize(x, mode)
+    ws = torch.zeros(ops.linear_workspace_bytes(M, N, K), dtype=torch.uint8, device=DEV)
+    y = ops.linear(x, w, mode, workspace=ws)
+    A, B = ops.mixfp4_dequantize(q).double(), ops.mixfp4_dequantize(w).double()
+    assert torch.all((y.double() - A @ B.T).abs() <= 1e-5 * (A.abs() @ B.abs().T))
+    header = 2048 * 4 + 256    # the maxima and s32 come first
+    assert torch.equal(ws[header:header + M * (K // 2)].view(M, K // 2), q.codes) == codes
