@@ -67,3 +67,31 @@ def test_linear_one_column_of_tiles(tiles, extra, N, K, mode, pad, codes):
     assert torch.all((y.double() - A @ B.T).abs() <= 1e-5 * (A.abs() @ B.abs().T))
     header = 2048 * 4 + 256    # the maxima and s32 come first
     assert torch.equal(ws[header:header + M * (K // 2)].view(M, K // 2), q.codes) == codes
+
+
+# The activations' maximum is reduced from one word per CTA of the first pass (456
+# on 152 SMs, 1216 beyond 2^23 blocks): the largest value in the blocks of the
+# first, the last and middle CTAs, at the tensor's ends and in later rounds.
+@pytest.mark.parametrize("M,N,K", [(2048, 600, 4096), (33000, 300, 4096)])
+def test_linear_finds_the_maximum_anywhere(M, N, K):
+    from paper_2605_31035_gb300 import ops, synth
+    g = torch.Generator(device=DEV).manual_seed(5)
+    x = (torch.randn(M, K, generator=g, device=DEV) * 0.01).to(torch.bfloat16)
+    w = ops.mixfp4_quantize(synth.weights(N, K, 8620, 0.02, 0.5).to(DEV))
+    B = ops.mixfp4_dequantize(w).double()
+    nblocks = M * K // 16
+    ctas = torch.cuda.get_device_properties(0).multi_processor_count * (8 if nblocks > 1 << 23 else 3)
+    for cta in (0, 1, 255, 256, 300, ctas - 1):
+        for rnd in (0, 2):
+            block = nblocks - 1 - (rnd * ctas * 256 + cta * 256 + 37)    # the pass reads from the end
+            if block < 0:
+                continue
+            r, c = divmod(block * 16 + 11, K)
+            old = x[r, c].clone()
+            x[r, c] = -100.0
+            rows = torch.tensor([r, (r + M // 2) % M], device=DEV)
+            q = ops.mixfp4_quantize(x)
+            A = ops.mixfp4_dequantize(ops.QTensor(q.codes[rows], q.scales[rows], q.tensor_scale)).double()
+            y = ops.linear(x, w)[rows].double()
+            assert torch.all((y - A @ B.T).abs() <= 1e-5 * (A.abs() @ B.abs().T)), (cta, rnd)
+            x[r, c] = old
