@@ -35,8 +35,8 @@
 // PFLOP/s).  Bound: the tensor pipe (91 % busy on 4096 x 14336 x 4096), on one
 // or two waves the launch, first loads and last drain, about 8 us.
 // Every pipeline wait is bounded; a wait that gives up records a status bit
-// (1 / 2 producers, 4 MMA waiting for a stage, 8 final drain, 16 / 32
-// decoders, 64 epilogue, 128 forwarder) and the CTA drains and exits.
+// (1 producers, 2 / 4 MMA waiting for an accumulator / a stage, 8 final drain,
+// 16 / 32 decoders, 64 epilogue, 128 forwarder) and the CTA drains and exits.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
@@ -280,7 +280,7 @@ gemm_f16a_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
         for (int kc = k0; kc < k1; ++kc, ++it) {
           const int s = it % kCodeStages;
           if (!mbar_wait(smem_u32(&bars->code_empty[s]), ((it / kCodeStages) & 1) ^ 1, abort_flag, kWaitLimitNs)) {
-            fail(2u);
+            fail(1u);
             ok = false;
             break;
           }

@@ -66,3 +66,20 @@ def test_shared_device_code_reads_coherently():
         assert "ld.global.nc" not in text, f
         if f.endswith(".cuh"):
             assert "__ldg" not in text, f
+
+
+# The status bits that the header documents: 1 a producer's wait, 2 / 4 the
+# MMA thread's for an accumulator or a stage, 8 its final drain.
+PIPELINED = [k for k in KERNELS if "fail(" in k[3]]
+
+
+@pytest.mark.parametrize("body", [k[3] for k in PIPELINED], ids=[k[1] for k in PIPELINED])
+def test_status_bits_name_their_role(body):
+    roles = re.split(r"(?:else )?if \(warp\b", body)[1:]
+    mma = [bool(re.search(r"\bmma_(f16|nvf4)\w*\s*\(", r)) for r in roles]
+    assert any(mma)
+    for r, issues_mma in zip(roles, mma):
+        bits = set(re.findall(r"fail\((\d+)u\)", r))
+        assert issues_mma or not bits & {"2", "4", "8"}
+        if "tma_load_2d" in r and not issues_mma:
+            assert bits <= {"1"}
