@@ -151,10 +151,10 @@ fewrows_prep_kernel(const uint8_t* codes, const uint8_t* scales, int M, int xr, 
                     uint8_t* __restrict__ sfa) {
   griddep_wait();
   griddep_launch_dependents();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int per_row = K / 32;
-  if (i >= xr * per_row) return;
-  const int r = i / per_row, c = i - r * per_row;
+  // Unsigned: 64 rows of K = 2^30 are 2^31 chunks.
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x, per_row = (uint32_t)K / 32;
+  if (i >= (uint32_t)xr * per_row) return;
+  const int r = (int)(i / per_row), c = (int)(i - (uint32_t)r * per_row);
   uint4 w = make_uint4(0u, 0u, 0u, 0u);
   uint32_t s4 = 0u;  // scales of the 64-K step this chunk lies in
   if (r < M) {

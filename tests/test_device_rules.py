@@ -83,3 +83,10 @@ def test_status_bits_name_their_role(body):
         assert issues_mma or not bits & {"2", "4", "8"}
         if "tma_load_2d" in r and not issues_mma:
             assert bits <= {"1"}
+
+
+@pytest.mark.parametrize("body", [k[3] for k in KERNELS], ids=[k[1] for k in KERNELS])
+def test_flat_indices_hold_the_largest_sizes(body):
+    """A flat index over all threads is not a signed 32-bit number: 64 rows of
+    K = 2^30, which the GEMMs take, are 2^31 chunks of 32."""
+    assert not re.search(r"\bint\s+\w+\s*=\s*(\(int\)\s*)?\(?\s*blockIdx\.x\s*\*", body)
