@@ -49,7 +49,8 @@
 //
 // Every pipeline wait is bounded; a wait that gives up records a status bit
 // (1 producer, 2 / 4 MMA thread, 8 final drain, 16 / 32 splitters, 64
-// epilogue) and the CTA drains and exits without storing more of C.
+// epilogue) and the CTA drains and exits without storing more of its output.  With
+// K in parts the sum kernel still runs, over parts that may not have been written.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>

@@ -32,8 +32,9 @@
 // Measured against the in-loop decode of gemm.cu (warm L2, batches, with the
 // decode pass of A): 2048 x 4096 x 4096 51.5 -> 43.3 us, 4096 x 14336 x 4096
 // 279 -> 241, 4096 x 4096 x 14336 298 -> 262, 8192^3 643 -> 557 us (1.97
-// PFLOP/s).  Bound: the tensor pipe (91 % busy on 4096 x 14336 x 4096), on one
-// or two waves the launch, first loads and last drain, about 8 us.
+// PFLOP/s).  Bound: the tensor pipe on many waves (83.6 % of active cycles at
+// 4096^3); on two (74.7 % at 2048 x 4096 x 4096) a stage's waits, commits and
+// decoder round beside it, and the launch, first loads and last drain, about 8 us.
 // Every pipeline wait is bounded; a wait that gives up records a status bit
 // (1 producers, 2 / 4 MMA waiting for an accumulator / a stage, 8 final drain,
 // 16 / 32 decoders, 64 epilogue, 128 forwarder) and the CTA drains and exits.
@@ -551,8 +552,11 @@ int64_t parts_bytes(int64_t M, int64_t N, int splits) {
 // 224, 450 at 160, 415 at 96; the tensor pipe alone is 2 n), so a width costs
 // its waves times that.  Two ways to use pairs that would idle:
 // - a partial last wave's K slices shared out over all pairs (stream-K: C rows
-//   zeroed, partial sums added), about 17000 cycles (memset, the lost launch
-//   overlap, one more drain and the adds; 15800 to 19800 over four shapes);
+//   zeroed, partial sums added), about 17000 cycles (the zeroing kernel, one more
+//   drain and the adds: 7.5 to 10 us over ten shapes.  256-wide tiles whole / split,
+//   L2 flushed, us: 2560 x 4096 x 4096 71.7 / 62.9, 3072 x 4096 x 4096 72.9 / 72.6,
+//   4096 x 4096 x 2304 59.5 / 61.5; at 4096^3 93.3 / 89.4, and 85.1 as whole 224-wide
+//   tiles, which the plan takes);
 // - where the tiles do not fill one wave, K cut into parts that are summed by
 //   sum_parts_kernel, if the caller's workspace holds the parts: about 8000
 //   cycles plus the parts' traffic.

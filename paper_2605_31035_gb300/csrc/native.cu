@@ -415,6 +415,10 @@ nvf4_gemm_kernel(const __grid_constant__ CUtensorMap tm_am, const __grid_constan
   }
 }
 
+// K slices a split last wave must save per pair.  Whole / split, L2 flushed, us, by the
+// slices saved: 2304^2 x 2048 38.1 / 36.7 (7.5), 3072 x 4096 x 4096 72.9 / 71.8 (7.6),
+// 4096 x 4096 x 2304 62.7 / 65.8 (5.7), 6144 x 6144 x 3072 132.4 / 136.6 (5.1), 4096^3
+// 91.3 / 89.2 (10.1), 2560 x 4096 x 4096 73.7 / 64.0 (14.3).
 constexpr int kMinStreamKGainSlices = 8;
 
 template <bool kARes, bool kBRes>
@@ -556,9 +560,6 @@ __device__ __forceinline__ uint32_t residual_scales(uint32_t sw) {
   asm("prmt.b32 %0, %1, %2, 0xBA98;" : "=r"(m) : "r"(sw), "r"(0u));
   return sw & m & 0x7F7F7F7Fu;
 }
-
-// Row r's four ue4m3 scales of K step j in the tiled layout of a 128-row tile.
-__device__ __forceinline__ uint32_t sf_offset(int r) { return (uint32_t)((r & 31) * 16 + (r >> 5) * 4); }
 
 __global__ void __launch_bounds__(kThreads, 1)
 nvf4_fewrows_kernel(const __grid_constant__ CUtensorMap tm_wc, const __grid_constant__ CUtensorMap tm_ws,
@@ -741,8 +742,8 @@ nvf4_fewrows_kernel(const __grid_constant__ CUtensorMap tm_wc, const __grid_cons
         const uint32_t swz = (uint32_t)(row & 7);
         {
           const uint32_t sw = lds32(sp + OWS + (uint32_t)row * 16 + (uint32_t)q4 * 4);
-          sts32(sp + OSFB + q4 * 512 + sf_offset(row), sw & 0x7F7F7F7Fu);
-          sts32(sp + OSFR + q4 * 512 + sf_offset(row), residual_scales(sw));
+          sts32(sp + OSFB + q4 * 512 + tiled_scale_row(row), sw & 0x7F7F7F7Fu);
+          sts32(sp + OSFR + q4 * 512 + tiled_scale_row(row), residual_scales(sw));
         }
         fence_proxy_async_smem();
         __syncwarp();
@@ -757,8 +758,8 @@ nvf4_fewrows_kernel(const __grid_constant__ CUtensorMap tm_wc, const __grid_cons
         for (int q = t; q < nx * 4; q += kXSplitWarps * 32) {  // scale word q % 4 of row q / 4
           const int row = q >> 2, j = q & 3;
           const uint32_t sw = lds32(sp + OXS + (uint32_t)row * 16 + (uint32_t)j * 4);
-          sts32(sp + OSFA + j * 512 + sf_offset(row), sw & 0x7F7F7F7Fu);
-          sts32(sp + OSFA + j * 512 + sf_offset(row + XR), residual_scales(sw));
+          sts32(sp + OSFA + j * 512 + tiled_scale_row(row), sw & 0x7F7F7F7Fu);
+          sts32(sp + OSFA + j * 512 + tiled_scale_row(row + XR), residual_scales(sw));
         }
         fence_proxy_async_smem();
         __syncwarp();
